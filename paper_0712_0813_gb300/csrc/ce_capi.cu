@@ -216,14 +216,9 @@ ce::DiagArgs<T> make_diag_args(const ce_sim* s, int raw_u) {
   return a;
 }
 
-int diag_blocks(const ce_sim* s) {
-  int64_t want = (s->S + 255) / 256;
-  return (int)(want < s->diag_blocks_max ? want : s->diag_blocks_max);
-}
-
 cudaError_t run_diag(const ce_sim* s, int raw_u) {
-  if (s->prec == CE_F32) return ce::launch_diag<float>(make_diag_args<float>(s, raw_u), diag_blocks(s), s->stream);
-  return ce::launch_diag<double>(make_diag_args<double>(s, raw_u), diag_blocks(s), s->stream);
+  if (s->prec == CE_F32) return ce::launch_diag<float>(make_diag_args<float>(s, raw_u), s->diag_blocks_max, s->stream);
+  return ce::launch_diag<double>(make_diag_args<double>(s, raw_u), s->diag_blocks_max, s->stream);
 }
 
 // Copy the aux block back and turn a latched device error into a return code.

@@ -1,0 +1,392 @@
+// ce_diag.cu -- the diagnostics pass: kinetic, gradient and potential energies
+// and the fields' moments in one sweep over f and w, reduced and turned into
+// the outputs by the launch's last block (one launch per read-out).
+//
+// Per site (arXiv:0712.0813 Sec. II outputs; the synchronised velocity is
+// that of site_u in ce_generic.cu):
+//   v_half = w + c f;  v(t_n) = v_half - dt/2 (lap f - dV/df + s f)
+//   a'(t_n) = a'_{n+1/2} - dt/2 a''_n;  u = v(t_n) - (a'(t_n)/a_n) f
+// With raw_u (start-up input) u is w itself.
+//
+// The pass reads f and w once (2 NF x sizeof(T) per site).  For FP32 storage HBM
+// bounds it, provided the FP64 pipe (two lanes per clock and SM: 64 cycles a warp
+// instruction and scheduler) stays out of it: a thread's partials stay in FP32 for
+// at most 16 sites and are then added, with the addition's rounding error kept
+// (add_to), to float pairs of 48 bits, which the lanes add the same way; only the
+// warps' sums become FP64.  The partials' own rounding (2^-24 over 16 sites) is what
+// limits the sums, as when they went to FP64 accumulators.  That flush, as a counter
+// test inside the site loop, was if-converted into 9 conversions and 9 FP64
+// additions a site (256^3, two fields: 606 us where the bytes take 40), and as a
+// loop of its own still took 202 us, half of it the warps' FP64 shuffle sums.
+// FP64 storage is bound by its FP64 arithmetic.
+#include <algorithm>
+#include <cstdint>
+
+#include "ce_device.cuh"
+#include "ce_internal.h"
+
+namespace ce {
+namespace {
+
+constexpr int kDiagThreads = 256;
+constexpr int kDiagWarps = kDiagThreads / 32;
+constexpr int kFlush = 16;   // sites a thread sums in T before adding to its running sums
+
+// How the lattice is cut into block tasks.  3D: a task is 32 x-sites by 8 rows
+// (one per warp, so the y-neighbours of the inner rows hit L1) swept along a
+// chunk of z; 2D: 256 x-sites swept along a chunk of y; 1D: 256 threads x 16
+// sites, strided.  Along the sweep the neighbours stay in registers.  Chunks of 16
+// (their end planes, read twice, hit L2), shorter where that leaves blocks without
+// a task: there one thread's sweep is pure latency.  Warp strips with the y- and
+// x-neighbours in registers and a plane of loads in flight (the column kernel's
+// layout) need half the loads but 164 registers: 217 against 142 us at 256^3.
+struct DiagTasks {
+  int nx, ny;      // x-segments (2D, 3D), row groups (3D)
+  int len;         // sites per task along the sweep
+  int64_t count;
+};
+
+DiagTasks diag_tasks(int dims, int64_t N, int64_t S, int blocks) {
+  DiagTasks t{1, 1, kFlush, 0};
+  if (dims == 1) {
+    t.count = (S + kDiagThreads * kFlush - 1) / (kDiagThreads * kFlush);
+    return t;
+  }
+  t.nx = (int)((N + (dims == 3 ? 31 : kDiagThreads - 1)) / (dims == 3 ? 32 : kDiagThreads));
+  t.ny = dims == 3 ? (int)((N + kDiagWarps - 1) / kDiagWarps) : 1;
+  for (t.len = kFlush; t.len > 4; t.len /= 2)
+    if ((int64_t)t.nx * t.ny * ((N + t.len - 1) / t.len) >= blocks / 2) break;
+  t.count = (int64_t)t.nx * t.ny * ((N + t.len - 1) / t.len);
+  return t;
+}
+
+// Per-launch scalars in the storage type.
+template <typename T>
+struct DiagScalars {
+  T idx2, half_dt, c, h, sterm;
+  T q[3];
+};
+
+template <typename T>
+__device__ __forceinline__ DiagScalars<T> diag_scalars(const DiagArgs<T>& p) {
+  DiagScalars<T> k;
+  const DevScalars sc = *p.sc;
+  k.idx2 = (T)p.inv_dx2;
+  k.half_dt = (T)(0.5 * p.dt);
+  k.c = (T)sc.c;
+  k.h = (p.expansion && !p.raw_u) ? (T)((sc.ap - 0.5 * p.dt * sc.app) / sc.a) : T(0);
+  k.sterm = (p.expansion && !p.raw_u) ? (T)sc.s : T(0);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) k.q[i] = (T)p.q[i];
+  return k;
+}
+
+// One site's terms added to part: [K_i (NF)][G_i (NF)][V][f_i - f_i(0) (NF)]
+// [(f_i - f_i(0))^2 (NF)].  nb[d][0] / nb[d][1]: the neighbours at +e_d / -e_d.
+template <typename T, int NF, int DIMS>
+__device__ __forceinline__ void diag_site(const DiagScalars<T>& k, int raw_u, const T (&f)[NF], const T (&w)[NF],
+                                          const T (&nb)[NF][DIMS][2], const T (&shift)[NF],
+                                          T (&part)[4 * NF + 1]) {
+  T dv[NF], vs;
+  model_dv<T, NF>(f, k.q, dv, vs);
+  part[2 * NF] += vs;
+#pragma unroll
+  for (int i = 0; i < NF; ++i) {
+    T lap = T(0);
+    if constexpr (sizeof(T) == 8) {   // fewer FP64 operations; its rounding is far below the sums'
+      T sum = nb[i][0][0] + nb[i][0][1];
+#pragma unroll
+      for (int d = 1; d < DIMS; ++d) sum += nb[i][d][0] + nb[i][d][1];
+      lap = fmaT(T(-2 * DIMS), f[i], sum);
+    } else {
+#pragma unroll
+      for (int d = 0; d < DIMS; ++d) lap += (nb[i][d][0] + nb[i][d][1]) - T(2) * f[i];
+    }
+#pragma unroll
+    for (int d = 0; d < DIMS; ++d) {
+      const T df = nb[i][d][0] - f[i];
+      part[NF + i] = fmaT(df, df, part[NF + i]);
+    }
+    T u = w[i];
+    if (!raw_u) {
+      const T vh = fmaT(k.c, f[i], w[i]);
+      const T F = fmaT(lap, k.idx2, -dv[i]) + k.sterm * f[i];
+      u = fmaT(-k.half_dt, F, vh) - k.h * f[i];
+    }
+    part[i] = fmaT(T(0.5) * u, u, part[i]);
+    const T df = f[i] - shift[i];
+    part[2 * NF + 1 + i] += df;
+    part[3 * NF + 1 + i] = fmaT(df, df, part[3 * NF + 1 + i]);
+  }
+}
+
+// hi + lo += x: the addition's rounding error (Knuth's TwoSum, exact) joins lo.
+__device__ __forceinline__ void add_to(float& hi, float& lo, float x) {
+  const float s = hi + x;
+  const float b = s - hi;
+  lo += (hi - (s - b)) + (x - b);
+  hi = s;
+}
+
+// A thread's running sums: FP64, or float pairs.  Partials of 2^100 and above,
+// infinities and NaN would leave the pairs' range: they go to the block's FP64
+// sums `big` in shared memory.
+template <typename T, int NV>
+struct RunningSums;
+template <int NV>
+struct RunningSums<double, NV> {
+  double v[NV];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) v[j] = 0.0;
+  }
+  __device__ __forceinline__ void add(const double (&part)[NV], double*) {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) v[j] += part[j];
+  }
+  __device__ __forceinline__ double warp_total(int j) { return warp_sum(v[j]); }
+};
+template <int NV>
+struct RunningSums<float, NV> {
+  float hi[NV], lo[NV];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) hi[j] = lo[j] = 0.f;
+  }
+  __device__ __forceinline__ void add(const float (&part)[NV], double* big) {
+    bool fits = true;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) fits = fits && fabsf(part[j]) < 0x1p100f;
+    if (__all_sync(0xffffffffu, fits)) {   // every lane of the warp is here
+#pragma unroll
+      for (int j = 0; j < NV; ++j) add_to(hi[j], lo[j], part[j]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < NV; ++j) atomicAdd(big + j, (double)part[j]);
+    }
+  }
+  __device__ __forceinline__ double warp_total(int j) {
+    float h = hi[j], l = lo[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      l += __shfl_down_sync(0xffffffffu, l, o);
+      add_to(h, l, __shfl_down_sync(0xffffffffu, h, o));
+    }
+    return (threadIdx.x & 31) == 0 ? (double)h + (double)l : 0.0;
+  }
+};
+
+// The launch's last block: combine the blocks' sums (warp k takes quantity k,
+// k + 8, ...; lane l takes blocks l, l + 32, ..., then a fixed shuffle tree) and
+// derive the outputs.
+template <typename T, int NF>
+__device__ __forceinline__ void diag_outputs(const DiagArgs<T>& p, int blocks) {
+  constexpr int NV = 4 * NF + 1;
+  __shared__ double tot[NV];
+  const int lane = threadIdx.x & 31;
+  for (int k = threadIdx.x >> 5; k < NV; k += kDiagWarps) {
+    double t = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < blocks; b += 32) t += __ldcg(p.partials + (int64_t)b * NV + k);
+    t = warp_sum(t);
+    if (lane == 0) tot[k] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  double* r = p.aux->result;
+  for (int k = 0; k < kResultLen; ++k) r[k] = 0.0;
+  const double invS = 1.0 / (double)p.S;
+  double K = 0.0, G = 0.0;
+  for (int i = 0; i < NF; ++i) {
+    r[R_K + i] = tot[i] * invS;
+    r[R_G + i] = tot[NF + i] * (0.5 * p.inv_dx2) * invS;
+    K += tot[i] * invS;
+    G += tot[NF + i] * (0.5 * p.inv_dx2) * invS;
+  }
+  const double V = tot[2 * NF] * invS;
+  const double E = K + G + V;
+  r[R_V] = V;
+  r[R_KTOT] = K;
+  r[R_GTOT] = G;
+  r[R_E] = E;
+  const DevScalars s = *p.sc;
+  const double ap_t = p.expansion ? s.ap - 0.5 * p.dt * s.app : 0.0;
+  r[R_A] = p.expansion ? s.a : 1.0;
+  r[R_AP] = ap_t;
+  r[R_RESID] = p.expansion ? fabs(ap_t * ap_t / p.kappa2 - E) / E : 0.0;
+  for (int i = 0; i < NF; ++i) {
+    const double m1 = tot[2 * NF + 1 + i] * invS;   // <f - f(0)>
+    const double m2 = tot[3 * NF + 1 + i] * invS;   // <(f - f(0))^2>
+    r[R_MEAN + i] = m1 + (double)p.f[i][0];
+    r[R_VAR + i] = m2 - m1 * m1;
+  }
+  if (!isfinite(E)) atomicCAS(&p.aux->status, CE_OK, CE_ENONFINITE);
+}
+
+template <typename T, int NF, int DIMS>
+__global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 1) k_diag(const DiagArgs<T> p, const DiagTasks tk) {
+  constexpr int NV = 4 * NF + 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t N = p.N;
+  const DiagScalars<T> k = diag_scalars(p);
+  const int raw_u = p.raw_u;
+  __shared__ double red[kDiagWarps][NV], big[NV];
+  __shared__ int s_last;
+  if (threadIdx.x < NV) big[threadIdx.x] = 0.0;
+  __syncthreads();
+  RunningSums<T, NV> acc;
+  acc.clear();
+  T shift[NF];
+#pragma unroll
+  for (int i = 0; i < NF; ++i) shift[i] = p.f[i][0];
+  if constexpr (DIMS == 1) {
+    for (int64_t task = blockIdx.x; task < tk.count; task += gridDim.x) {
+      T part[NV];
+#pragma unroll
+      for (int j = 0; j < NV; ++j) part[j] = T(0);
+      const int64_t s0 = task * (kDiagThreads * kFlush) + threadIdx.x;
+#pragma unroll 4
+      for (int r = 0; r < kFlush; ++r) {
+        const int64_t s = s0 + r * kDiagThreads;
+        if (s >= p.S) break;
+        T f[NF], w[NF], nb[NF][1][2];
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+          f[i] = __ldg(p.f[i] + s);
+          w[i] = __ldg(p.w[i] + s);
+          nb[i][0][0] = __ldg(p.f[i] + (s == N - 1 ? 0 : s + 1));
+          nb[i][0][1] = __ldg(p.f[i] + (s == 0 ? N - 1 : s - 1));
+        }
+        diag_site<T, NF, 1>(k, raw_u, f, w, nb, shift, part);
+      }
+      __syncwarp();
+      acc.add(part, big);
+    }
+  } else {
+    const int64_t plane = DIMS == 3 ? N * N : N;               // stride of the sweep axis
+    for (int64_t task = blockIdx.x; task < tk.count; task += gridDim.x) {
+      // the lane's column: (x, y) in 3D, x in 2D; columns past the lattice's end
+      // repeat its last one and add nothing
+      const int xs = (int)(task % tk.nx);
+      const int64_t rest = task / tk.nx;
+      const int n = (int)N;                                    // sides below 2^17
+      int x, y = 0, chunk;
+      if constexpr (DIMS == 3) {
+        x = xs * 32 + lane;
+        y = (int)(rest % tk.ny) * kDiagWarps + warp;
+        chunk = (int)(rest / tk.ny);
+      } else {
+        x = xs * kDiagThreads + threadIdx.x;
+        chunk = (int)rest;
+      }
+      const bool site = x < n && y < n;
+      x = min(x, n - 1);
+      y = min(y, n - 1);
+      // offsets in a plane, added to the plane's (uniform) base
+      const uint32_t o = (uint32_t)y * (uint32_t)n + x;
+      const uint32_t oxp = x == n - 1 ? o - (n - 1) : o + 1, oxm = x == 0 ? o + (n - 1) : o - 1;
+      const uint32_t oyp = y == n - 1 ? o - (n - 1) * n : o + n, oym = y == 0 ? o + (n - 1) * n : o - n;
+      const int z0 = chunk * tk.len, z1 = min(z0 + tk.len, n);
+      T fm[NF], fc[NF], part[NV];
+#pragma unroll
+      for (int i = 0; i < NF; ++i) {
+        fm[i] = __ldg(p.f[i] + (z0 == 0 ? n - 1 : z0 - 1) * plane + o);
+        fc[i] = __ldg(p.f[i] + z0 * plane + o);
+      }
+#pragma unroll
+      for (int j = 0; j < NV; ++j) part[j] = T(0);
+      constexpr int kUnroll = sizeof(T) == 8 ? 1 : (NF <= 2 ? 2 : 4);
+#pragma unroll kUnroll
+      for (int z = z0; z < z1; ++z) {
+        const int64_t here = z * plane, next = (z + 1 == n ? 0 : z + 1) * plane;
+        T w[NF], nb[NF][DIMS][2], fn[NF];
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+          const T* fz = p.f[i] + here;
+          fn[i] = __ldg(p.f[i] + next + o);
+          w[i] = __ldg(p.w[i] + here + o);
+          nb[i][0][0] = __ldg(fz + oxp);
+          nb[i][0][1] = __ldg(fz + oxm);
+          if constexpr (DIMS == 3) {
+            nb[i][1][0] = __ldg(fz + oyp);
+            nb[i][1][1] = __ldg(fz + oym);
+          }
+          nb[i][DIMS - 1][0] = fn[i];
+          nb[i][DIMS - 1][1] = fm[i];
+        }
+        diag_site<T, NF, DIMS>(k, raw_u, fc, w, nb, shift, part);
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+          fm[i] = fc[i];
+          fc[i] = fn[i];
+        }
+      }
+      if (!site) {   // the whole warp takes part in the addition
+#pragma unroll
+        for (int j = 0; j < NV; ++j) part[j] = T(0);
+      }
+      __syncwarp();
+      acc.add(part, big);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    const double v = acc.warp_total(j);
+    if (lane == 0) red[warp][j] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < NV) {
+    double t = big[threadIdx.x];
+    for (int w = 0; w < kDiagWarps; ++w) t += red[w][threadIdx.x];
+    p.partials[(int64_t)blockIdx.x * NV + threadIdx.x] = t;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&p.aux->counter_diag, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  diag_outputs<T, NF>(p, gridDim.x);
+  if (threadIdx.x == 0) p.aux->counter_diag = 0u;
+}
+
+// A grid that is resident as a whole (at most `cap` blocks): tasks are strided.
+template <typename T, int NF, int DIMS>
+cudaError_t launch_diag_dims(const DiagArgs<T>& a, int cap, cudaStream_t st) {
+  int per_sm = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_diag<T, NF, DIMS>, kDiagThreads, 0) != cudaSuccess ||
+      per_sm < 1) {
+    cudaGetLastError();
+    per_sm = 1;
+  }
+  cap = std::min(cap, per_sm * sm_count(-1));
+  const DiagTasks tk = diag_tasks(DIMS, a.N, a.S, cap);
+  const int blocks = (int)std::min<int64_t>(tk.count, cap);
+  k_diag<T, NF, DIMS><<<blocks, kDiagThreads, 0, st>>>(a, tk);
+  return cudaGetLastError();
+}
+
+template <typename T, int NF>
+cudaError_t launch_diag_nf(const DiagArgs<T>& a, int cap, cudaStream_t st) {
+  switch (a.dims) {
+    case 1: return launch_diag_dims<T, NF, 1>(a, cap, st);
+    case 2: return launch_diag_dims<T, NF, 2>(a, cap, st);
+    default: return launch_diag_dims<T, NF, 3>(a, cap, st);
+  }
+}
+
+}  // namespace
+
+template <typename T>
+cudaError_t launch_diag(const DiagArgs<T>& a, int cap, cudaStream_t st) {
+  switch (a.nf) {
+    case 1: return launch_diag_nf<T, 1>(a, cap, st);
+    case 2: return launch_diag_nf<T, 2>(a, cap, st);
+    case 3: return launch_diag_nf<T, 3>(a, cap, st);
+    default: return launch_diag_nf<T, 4>(a, cap, st);
+  }
+}
+template cudaError_t launch_diag<float>(const DiagArgs<float>&, int, cudaStream_t);
+template cudaError_t launch_diag<double>(const DiagArgs<double>&, int, cudaStream_t);
+
+}  // namespace ce

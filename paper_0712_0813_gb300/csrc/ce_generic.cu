@@ -1,8 +1,8 @@
 // ce_generic.cu -- the generic step (any dimension, any N >= 3): the fused
 // one-thread-per-site kernel, its vectorised 1D form, and a two-pass form for
 // FP64 in 2D/3D (g written once, then the stencil; FP64 is rate-bound); plus
-// the diagnostics pass, the start-up scalar kernel and the host<->device
-// conversion kernels of libclusterlat.
+// the synchronised-velocity download, the start-up scalar kernel and the
+// host<->device conversion kernels of libclusterlat.
 //
 // The fused step (arXiv:0712.0813 Sec. III staggered leapfrog) per site x and
 // field i, with state (f_n, w_n) and v_{n+1/2} = w_n + c_n f_n:
@@ -346,169 +346,40 @@ template cudaError_t launch_step_generic<float>(const StepArgs<float>&, int, cud
 template cudaError_t launch_step_generic<double>(const StepArgs<double>&, int, cudaStream_t);
 
 // ---------------------------------------------------------------------------
-// Diagnostics: u(t_n), energies and moments in FP64 (on demand, not per step).
+// The synchronised velocity u(t_n) at a site (downloads; the sums of ce_diag.cu
+// form it the same way):
 //   v_half = w + c f;  v(t_n) = v_half - dt/2 (lap f - dV/df + s f)
 //   a'(t_n) = a'_{n+1/2} - dt/2 a''_n;  u = v(t_n) - (a'(t_n)/a_n) f
-// With raw_u (start-up input) u is w itself.
-
-// Per-site quantities in the compute type C: f, u(t_n), the forward-difference
-// gradient term sum_d (f(x+e_d) - f(x))^2 and V(f).  The sums (k_diag) use C =
-// the storage type, with per-thread partials in C folded into FP64 every 16
-// sites as in the step kernels: for FP32 storage the inputs carry 2^-24
-// relative rounding already, and FP64 per-site arithmetic (one conversion per
-// neighbour load) made the pass bound by GB300's FP64 rate.  The synchronised
-// velocity download (k_sync_u_range) uses C = the storage type as well (its
-// FP64 form made the download of a 1024^3 FP32 lattice FP64-bound: 0.32 s
-// against 0.20 s for the staggered velocity) and converts the result.
-template <typename T, typename C, int NF, int DIMS>
-__device__ __forceinline__ void site_u(const DiagArgs<T>& p, int64_t s, const SiteWalk<DIMS>& at,
-                                       C (&fv)[NF], C (&u)[NF], C (&g2)[NF], C& vsite) {
+// in the storage type: in FP64 the download of a 1024^3 FP32 lattice was bound by
+// GB300's FP64 rate (0.32 s against 0.20 s for the staggered velocity).
+template <typename T, int NF, int DIMS>
+__device__ __forceinline__ void site_u(const DiagArgs<T>& p, int64_t s, const SiteWalk<DIMS>& at, T (&u)[NF]) {
   int64_t nb[2 * DIMS];
   neighbours<DIMS>(s, at, p.N, nb);
-  C lap[NF];
-  const C idx2 = (C)p.inv_dx2;
+  T fv[NF], lap[NF], dv[NF], vsite;
+  const T idx2 = (T)p.inv_dx2;
 #pragma unroll
   for (int i = 0; i < NF; ++i) {
     const T* fi = p.f[i];
-    fv[i] = (C)fi[s];
-    C acc = C(0), gg = C(0);
+    fv[i] = fi[s];
+    T acc = T(0);
 #pragma unroll
-    for (int d = 0; d < DIMS; ++d) {
-      const C fp = (C)fi[nb[2 * d]], fm = (C)fi[nb[2 * d + 1]];
-      acc += (fp + fm) - C(2) * fv[i];
-      gg += (fp - fv[i]) * (fp - fv[i]);
-    }
+    for (int d = 0; d < DIMS; ++d) acc += (fi[nb[2 * d]] + fi[nb[2 * d + 1]]) - T(2) * fv[i];
     lap[i] = acc * idx2;
-    g2[i] = gg;
   }
-  C dv[NF];
-  C q[3] = {(C)p.q[0], (C)p.q[1], (C)p.q[2]};
-  model_dv<C, NF>(fv, q, dv, vsite);
-  if (p.raw_u) {
-#pragma unroll
-    for (int i = 0; i < NF; ++i) u[i] = (C)p.w[i][s];
-    return;
-  }
+  T q[3] = {(T)p.q[0], (T)p.q[1], (T)p.q[2]};
+  model_dv<T, NF>(fv, q, dv, vsite);
   const DevScalars sc = *p.sc;
-  const C h = p.expansion ? (C)((sc.ap - 0.5 * p.dt * sc.app) / sc.a) : C(0);
-  const C sterm = p.expansion ? (C)sc.s : C(0);
-  const C half_dt = (C)(0.5 * p.dt);
+  const T h = p.expansion ? (T)((sc.ap - 0.5 * p.dt * sc.app) / sc.a) : T(0);
+  const T sterm = p.expansion ? (T)sc.s : T(0);
+  const T half_dt = (T)(0.5 * p.dt);
   const T cT = (T)sc.c;
 #pragma unroll
   for (int i = 0; i < NF; ++i) {
-    const T vh = fmaT(cT, p.f[i][s], p.w[i][s]);
-    const C vsync = (C)vh - half_dt * (lap[i] - dv[i] + sterm * fv[i]);
+    const T vh = fmaT(cT, fv[i], p.w[i][s]);
+    const T vsync = vh - half_dt * (lap[i] - dv[i] + sterm * fv[i]);
     u[i] = vsync - h * fv[i];
   }
-}
-
-// partial layout per block: [K_i (NF)][G_i (NF)][V][sum(f_i - f_i(0)) (NF)][sum (f_i - f_i(0))^2 (NF)]
-template <typename T, int NF, int DIMS>
-__global__ void __launch_bounds__(256) k_diag(const DiagArgs<T> p) {
-  constexpr int NV = 4 * NF + 1;
-  double acc[NV];
-  T part[NV];   // per-thread partials in the storage type, folded into acc every 16 sites
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    acc[k] = 0.0;
-    part[k] = T(0);
-  }
-  T shift[NF];
-#pragma unroll
-  for (int i = 0; i < NF; ++i) shift[i] = p.f[i][0];
-  int since_flush = 0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t s0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  SiteWalk<DIMS> at;
-  at.init(s0, stride, p.N);
-  for (int64_t s = s0; s < p.S; s += stride, at.advance(p.N)) {
-    T fv[NF], u[NF], g2[NF], vs;
-    site_u<T, T, NF, DIMS>(p, s, at, fv, u, g2, vs);
-#pragma unroll
-    for (int i = 0; i < NF; ++i) {
-      part[i] += T(0.5) * u[i] * u[i];
-      part[NF + i] += g2[i];
-      const T df = fv[i] - shift[i];
-      part[2 * NF + 1 + i] += df;
-      part[3 * NF + 1 + i] += df * df;
-    }
-    part[2 * NF] += vs;
-    if (++since_flush == 16) {
-#pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        acc[k] += (double)part[k];
-        part[k] = T(0);
-      }
-      since_flush = 0;
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < NV; ++k) acc[k] += (double)part[k];
-  __shared__ double red[8][NV];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const double v = warp_sum(acc[k]);
-    if (lane == 0) red[warp][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < NV) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w][threadIdx.x];
-    p.partials[(int64_t)blockIdx.x * NV + threadIdx.x] = t;
-  }
-}
-
-// One block of one warp per quantity: combine the diag partials (lane l takes
-// blocks l, l + 32, ..., then a fixed shuffle tree) and derive the outputs.
-template <int NF>
-__global__ void k_diag_finalize(const double* partials, int blocks, DevAux* aux, int64_t S,
-                                double half_inv_dx2, double dt, double kappa2, int expansion,
-                                const DevScalars* sc) {
-  constexpr int NV = 4 * NF + 1;
-  __shared__ double tot[NV];
-  const int lane = threadIdx.x & 31;
-  for (int k = threadIdx.x >> 5; k < NV; k += blockDim.x >> 5) {
-    double t = 0.0;
-    for (int b = lane; b < blocks; b += 32) t += partials[(int64_t)b * NV + k];
-    t = warp_sum(t);
-    if (lane == 0) tot[k] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  double* r = aux->result;
-  for (int k = 0; k < kResultLen; ++k) r[k] = 0.0;
-  const double invS = 1.0 / (double)S;
-  double K = 0.0, G = 0.0;
-  for (int i = 0; i < NF; ++i) {
-    r[R_K + i] = tot[i] * invS;
-    r[R_G + i] = tot[NF + i] * half_inv_dx2 * invS;
-    K += r[R_K + i];
-    G += r[R_G + i];
-  }
-  r[R_V] = tot[2 * NF] * invS;
-  r[R_KTOT] = K;
-  r[R_GTOT] = G;
-  const double E = K + G + r[R_V];
-  r[R_E] = E;
-  const DevScalars s = *sc;
-  const double ap_t = expansion ? s.ap - 0.5 * dt * s.app : 0.0;
-  r[R_A] = expansion ? s.a : 1.0;
-  r[R_AP] = ap_t;
-  r[R_RESID] = expansion ? fabs(ap_t * ap_t / kappa2 - E) / E : 0.0;
-  for (int i = 0; i < NF; ++i) {
-    const double m1 = tot[2 * NF + 1 + i] * invS;   // <f - shift>
-    const double m2 = tot[3 * NF + 1 + i] * invS;   // <(f - shift)^2>
-    r[R_MEAN + i] = m1;                             // k_mean_shift adds the shift back
-    r[R_VAR + i] = m2 - m1 * m1;
-  }
-  if (!isfinite(E)) atomicCAS(&aux->status, CE_OK, CE_ENONFINITE);
-}
-
-template <typename T, int NF>
-__global__ void k_mean_shift(DevAux* aux, const T* f0, const T* f1, const T* f2, const T* f3) {
-  const T* fs[4] = {f0, f1, f2, f3};
-  for (int i = 0; i < NF; ++i) aux->result[R_MEAN + i] += (double)fs[i][0];
 }
 
 template <typename T, int NF, int DIMS>
@@ -519,43 +390,12 @@ __global__ void __launch_bounds__(256) k_sync_u_range(const DiagArgs<T> p) {
   at.init(p.s0 + k0, stride, p.N);
   for (int64_t k = k0; k < p.count; k += stride, at.advance(p.N)) {
     const int64_t s = p.s0 + k;
-    T fv[NF], u[NF], g2[NF], vs;
-    site_u<T, T, NF, DIMS>(p, s, at, fv, u, g2, vs);
+    T u[NF];
+    site_u<T, NF, DIMS>(p, s, at, u);
 #pragma unroll
     for (int i = 0; i < NF; ++i) p.u_out[(int64_t)i * p.count + k] = (double)u[i];
   }
 }
-
-template <typename T, int NF>
-static cudaError_t launch_diag_nf(const DiagArgs<T>& a, int blocks, cudaStream_t st) {
-  switch (a.dims) {
-    case 1: k_diag<T, NF, 1><<<blocks, 256, 0, st>>>(a); break;
-    case 2: k_diag<T, NF, 2><<<blocks, 256, 0, st>>>(a); break;
-    default: k_diag<T, NF, 3><<<blocks, 256, 0, st>>>(a); break;
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const double dx2inv = a.inv_dx2;
-  k_diag_finalize<NF><<<1, 32 * (4 * NF + 1), 0, st>>>(a.partials, blocks, a.aux, a.S, 0.5 * dx2inv, a.dt, a.kappa2,
-                                         a.expansion, a.sc);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_mean_shift<T, NF><<<1, 1, 0, st>>>(a.aux, a.f[0], a.f[NF > 1 ? 1 : 0], a.f[NF > 2 ? 2 : 0],
-                                       a.f[NF > 3 ? 3 : 0]);
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_diag(const DiagArgs<T>& a, int blocks, cudaStream_t st) {
-  switch (a.nf) {
-    case 1: return launch_diag_nf<T, 1>(a, blocks, st);
-    case 2: return launch_diag_nf<T, 2>(a, blocks, st);
-    case 3: return launch_diag_nf<T, 3>(a, blocks, st);
-    default: return launch_diag_nf<T, 4>(a, blocks, st);
-  }
-}
-template cudaError_t launch_diag<float>(const DiagArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_diag<double>(const DiagArgs<double>&, int, cudaStream_t);
 
 template <typename T, int NF>
 static cudaError_t launch_sync_nf(const DiagArgs<T>& a, cudaStream_t st) {

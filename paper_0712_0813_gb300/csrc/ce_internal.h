@@ -52,7 +52,7 @@ struct DevAux {
   DevScalars slot[2];
   int status;              // CE_OK or the first device-side error code
   unsigned int counter;    // last-block-done counter of the step reduction
-  unsigned int counter_diag;
+  unsigned int counter_diag;   // the same for the diagnostics pass
   int pad;
   double result[kResultLen];
 };
@@ -113,7 +113,8 @@ struct DiagArgs {
 
 // ---- launchers (return cudaError_t of the launch) -------------------------
 template <typename T> cudaError_t launch_step_generic(const StepArgs<T>& a, int blocks, cudaStream_t st);
-template <typename T> cudaError_t launch_diag(const DiagArgs<T>& a, int blocks, cudaStream_t st);
+// `cap`: most blocks the grid may have (partials holds 4 nf + 1 doubles for each).
+template <typename T> cudaError_t launch_diag(const DiagArgs<T>& a, int cap, cudaStream_t st);
 template <typename T> cudaError_t launch_sync_u_range(const DiagArgs<T>& a, cudaStream_t st);
 cudaError_t launch_init_scalars(DevAux* aux, int cur, int expansion, double dt, double kappa2,
                                 cudaStream_t st);
