@@ -72,10 +72,11 @@ extern "C" {
 #define CE_KERNEL_AUTO    0 /* FP32: z-sweep kernel where it applies; else the
                                row kernel for 2D sides >= 512 and 3D sides >= 256
                                it takes; else the column kernel (3D) or the
-                               line-sweep kernel (2D sides >= 320); else generic.  FP64: generic (its two-pass
-                               form), or the z-sweep kernel when plan hints
+                               line-sweep kernel (2D sides >= 320); else generic.  FP64: generic (the force in
+                               integer arithmetic), or the z-sweep kernel when plan hints
                                (tile_rows, stages, zchunks) are given          */
-#define CE_KERNEL_GENERIC 1 /* one thread per site, any d and N              */
+#define CE_KERNEL_GENERIC 1 /* any d and N: one thread per site (FP32), strips of
+                               30 sites with the force in integers (FP64)      */
 #define CE_KERNEL_SWEEP   2 /* 3D z-sweep kernel (CE_EINVAL if it does not apply) */
 #define CE_KERNEL_ROWS    3 /* the batched row-sweep kernel on this one lattice:
                                any d, N a multiple of 4 (FP32) / 2 (FP64)      */

@@ -158,7 +158,8 @@ cudaError_t launch_one_step(const ce_sim* s, int in, bool half_kick) {
   if (s->kernel == CE_KERNEL_PLANES)
     return s->dims == 3 ? ce::launch_step_cols<T>(a, s->cols, s->stream)
                         : ce::launch_step_lines<T>(a, s->lines, s->stream);
-  return ce::launch_step_generic<T>(a, s->generic_blocks, s->stream);
+  if constexpr (sizeof(T) == 8) return ce::launch_step_fx(a, s->fx, s->stream);
+  else return ce::launch_step_generic(a, s->generic_blocks, s->stream);
 }
 
 cudaError_t step_once(const ce_sim* s, int in, bool half_kick) {
@@ -379,11 +380,11 @@ int ce_create(const ce_config* cfg, ce_sim** out) {
   // Automatic choice.  FP32: the z-sweep kernel where it applies, else the row
   // kernel for the 2D and 3D lattices it takes from the sides above, else the
   // column kernel (3D) or the line-sweep kernel (2D) for odd and small sides,
-  // else (1D lattices, small 2D sides) the generic kernel.  FP64 is bound by the FP64 rate, and there
-  // the generic kernel's two-pass form (each site's g formed once) measured
-  // faster than both the z-sweep kernel (256^3: 1090 against 1141 us, tuned
-  // plan) and the row kernel (288^3: 1540 against 2967 us): the generic kernel,
-  // unless the caller gave z-sweep plan hints.
+  // else (1D lattices, small 2D sides) the generic kernel.  FP64, which GB300's
+  // two FP64 lanes per clock and SM would bound: the kernels that form the force
+  // in integers (ce_fx64.cu, under CE_KERNEL_GENERIC; 256^3: 596 us against 1141
+  // for the tuned z-sweep kernel and 2967 at 288^3 for the row kernel), unless the
+  // caller gave z-sweep plan hints.
   const bool sweep_hinted = cfg->tile_rows != 0 || cfg->stages != 0 || cfg->zchunks != 0;
   const bool rows_auto = rows_ok && cfg->precision == CE_F32 && cfg->dims >= 2 &&
                          cfg->N >= (cfg->dims == 3 ? kRowsMinN3 : kRowsMinN2);
@@ -443,6 +444,12 @@ int ce_create(const ce_config* cfg, ce_sim** out) {
     s->lines = ce::lines_plan(s->N, s->nf, s->prec, s->sms);
     planes_blocks = (int64_t)s->lines.gx * s->lines.gy;
   }
+  int64_t fx_blocks = 0;
+  if (s->prec == CE_F64) {   // also the fallback of the other kernels' set-up, and the row kernel's start-up
+    s->fx = ce::fx_plan(s->dims, s->N, s->nf, s->sms);
+    fx_blocks = (int64_t)s->fx.gx * s->fx.gy;
+  }
+  planes_blocks = std::max(planes_blocks, fx_blocks);
   int64_t nblk = std::max<int64_t>(std::max<int64_t>(s->generic_blocks, std::max(sweep_blocks, planes_blocks)), 1);
   int64_t plen = std::max<int64_t>(2 * nblk, (int64_t)s->diag_blocks_max * 17);
   s->partials = static_cast<double*>(dalloc(s, (size_t)plen * 8));

@@ -1,7 +1,6 @@
-// ce_generic.cu -- the generic step (any dimension, any N >= 3): the fused
-// one-thread-per-site kernel, its vectorised 1D form, and a two-pass form for
-// FP64 in 2D/3D (g written once, then the stencil; FP64 is rate-bound); plus
-// the synchronised-velocity download, the start-up scalar kernel and the
+// ce_generic.cu -- the generic FP32 step (any dimension, any N >= 3; FP64 has its
+// own, ce_fx64.cu): the fused one-thread-per-site kernel and its vectorised 1D
+// form; plus the synchronised-velocity download, the start-up scalar kernel and the
 // host<->device conversion kernels of libclusterlat.
 //
 // The fused step (arXiv:0712.0813 Sec. III staggered leapfrog) per site x and
@@ -171,66 +170,6 @@ __global__ void __launch_bounds__(kGenericThreads) k_step_generic(const StepArgs
   if (p.update_scalars) finish_step_block(p, (double)g2acc + (double)g2loc, (double)vacc + (double)vloc);
 }
 
-// FP64 in 2D and 3D, two passes.  In FP64 the step is bound by GB300's FP64
-// rate, and the one-pass kernel forms g = f + dt (w + c f) again for every
-// neighbour that reads it (2d + 1 times per site).  Pass 1 writes each site's g
-// once, into f_out (which holds g after the step anyway), and v = w + c f into
-// w_out (which pass 2 overwrites at the same site, in the same thread); pass 2
-// reads the neighbours' g and the site's v from there, sums the 2d neighbours
-// once and takes the gradient energy by summation by parts on the periodic lattice,
-//   sum_x sum_d (g(x+e_d) - g(x))^2 = -sum_x g(x) raw(x),
-//   raw(x) = sum_d (g(x+e_d) + g(x-e_d)) - 2d g(x)
-// (exact in exact arithmetic; the cancellation costs ~1e-12 of G in FP64, which
-// enters only a'').  About 16 FP64 operations per field and site instead of ~33.
-template <int NF>
-__global__ void __launch_bounds__(kGenericThreads) k_drift_g(const StepArgs<double> p) {
-  const double c = p.sc_in->c, dd = p.dt_drift;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < p.S; s += stride) {
-#pragma unroll
-    for (int i = 0; i < NF; ++i) {
-      const double f = p.f_in[i][s];
-      const double v = fma(c, f, p.w_in[i][s]);
-      p.w_out[i][s] = v;
-      p.f_out[i][s] = fma(dd, v, f);
-    }
-  }
-}
-
-template <int NF, int DIMS>
-__global__ void __launch_bounds__(kGenericThreads) k_kick_from_g(const StepArgs<double> p) {
-  const double kk = p.dt_kick, idx2 = p.inv_dx2;
-  const int64_t N = p.N, S = p.S;
-  double q[3] = {p.q[0], p.q[1], p.q[2]};
-  double grad2 = 0.0, pot = 0.0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t s0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  SiteWalk<DIMS> at;
-  at.init(s0, stride, N);
-  for (int64_t s = s0; s < S; s += stride, at.advance(N)) {
-    int64_t nb[2 * DIMS];
-    neighbours<DIMS>(s, at, N, nb);
-    double g[NF], lap[NF];
-#pragma unroll
-    for (int i = 0; i < NF; ++i) {
-      const double* gi = p.f_out[i];
-      g[i] = gi[s];
-      double nsum = gi[nb[0]] + gi[nb[1]];
-#pragma unroll
-      for (int d = 1; d < DIMS; ++d) nsum += gi[nb[2 * d]] + gi[nb[2 * d + 1]];
-      const double raw = fma(-2.0 * DIMS, g[i], nsum);
-      lap[i] = raw * idx2;
-      grad2 = fma(-g[i], raw, grad2);
-    }
-    double dv[NF], vs;
-    model_dv<double, NF>(g, q, dv, vs);
-    pot += vs;
-#pragma unroll
-    for (int i = 0; i < NF; ++i) p.w_out[i][s] = fma(kk, lap[i] - dv[i], p.w_out[i][s]);
-  }
-  if (p.update_scalars) finish_step_block(p, grad2, pot);
-}
-
 // One site s of a 1D lattice with the arithmetic of step1d_group (the sites
 // past the last whole 16-byte group of a side that is not a multiple of it).
 template <typename T, int NF>
@@ -315,35 +254,14 @@ static cudaError_t launch_generic_nf(const StepArgs<T>& a, int blocks, cudaStrea
   return cudaGetLastError();
 }
 
-template <int NF>
-static cudaError_t launch_two_pass_nf(const StepArgs<double>& a, int blocks, cudaStream_t st) {
-  k_drift_g<NF><<<blocks, kGenericThreads, 0, st>>>(a);
-  if (a.dims == 2) k_kick_from_g<NF, 2><<<blocks, kGenericThreads, 0, st>>>(a);
-  else k_kick_from_g<NF, 3><<<blocks, kGenericThreads, 0, st>>>(a);
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_step_generic(const StepArgs<T>& a, int blocks, cudaStream_t st) {
-  if constexpr (sizeof(T) == 8) {
-    if (a.dims >= 2) {
-      switch (a.nf) {
-        case 1: return launch_two_pass_nf<1>(a, blocks, st);
-        case 2: return launch_two_pass_nf<2>(a, blocks, st);
-        case 3: return launch_two_pass_nf<3>(a, blocks, st);
-        default: return launch_two_pass_nf<4>(a, blocks, st);
-      }
-    }
-  }
+cudaError_t launch_step_generic(const StepArgs<float>& a, int blocks, cudaStream_t st) {
   switch (a.nf) {
-    case 1: return launch_generic_nf<T, 1>(a, blocks, st);
-    case 2: return launch_generic_nf<T, 2>(a, blocks, st);
-    case 3: return launch_generic_nf<T, 3>(a, blocks, st);
-    default: return launch_generic_nf<T, 4>(a, blocks, st);
+    case 1: return launch_generic_nf<float, 1>(a, blocks, st);
+    case 2: return launch_generic_nf<float, 2>(a, blocks, st);
+    case 3: return launch_generic_nf<float, 3>(a, blocks, st);
+    default: return launch_generic_nf<float, 4>(a, blocks, st);
   }
 }
-template cudaError_t launch_step_generic<float>(const StepArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_step_generic<double>(const StepArgs<double>&, int, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // The synchronised velocity u(t_n) at a site (downloads; the sums of ce_diag.cu

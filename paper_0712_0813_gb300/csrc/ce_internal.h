@@ -112,7 +112,7 @@ struct DiagArgs {
 };
 
 // ---- launchers (return cudaError_t of the launch) -------------------------
-template <typename T> cudaError_t launch_step_generic(const StepArgs<T>& a, int blocks, cudaStream_t st);
+cudaError_t launch_step_generic(const StepArgs<float>& a, int blocks, cudaStream_t st);
 // `cap`: most blocks the grid may have (partials holds 4 nf + 1 doubles for each).
 template <typename T> cudaError_t launch_diag(const DiagArgs<T>& a, int cap, cudaStream_t st);
 template <typename T> cudaError_t launch_sync_u_range(const DiagArgs<T>& a, cudaStream_t st);
@@ -166,6 +166,12 @@ struct LinesPlan {
 LinesPlan lines_plan(int64_t N, int nf, int prec, int sms);
 template <typename T> cudaError_t launch_step_lines(const StepArgs<T>& a, const LinesPlan& plan,
                                                     cudaStream_t st);
+// The FP64 step with the force in integer arithmetic (any dimension and side).
+struct FxPlan {
+  int nstrips, gx, gy, len;
+};
+FxPlan fx_plan(int dims, int64_t N, int nf, int sms);
+cudaError_t launch_step_fx(const StepArgs<double>& a, const FxPlan& plan, cudaStream_t st);
 namespace sweep {
 cudaError_t launch_f32(int variant, const StepArgs<float>& a, const SweepMaps& m, dim3 grid, size_t smem,
                        cudaStream_t st);
@@ -208,6 +214,7 @@ struct ce_sim {
   ce::SweepPlan plan{};
   ce::ColsPlan cols{};
   ce::LinesPlan lines{};
+  ce::FxPlan fx{};             // FP64 handles on CE_KERNEL_GENERIC
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // kGraphSteps steps starting from buffer set 0 / 1
   bool graphs_ok = true;
   int64_t bytes = 0;
