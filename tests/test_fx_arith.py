@@ -15,8 +15,10 @@ compared with quad precision (CPU; no GPU needed):
 * the energy term, the sum over the fields of g times such a sum, is within 2^-53 of
   itself + the same errors times |g| + one unit a field for the product (a unit of
   it is at most 2^-56 of |g| times the stencil's largest value) + (nf + 1) half
-  units of the common grid, up to eight times as coarse; and its mean error,
-  which the sum over a lattice would carry, is within 2^-57 of its terms' sizes.
+  units of the common grid, up to eight times as coarse as the coarsest of those
+  units and of 4 dx^2 V's (at most 2^-57 of it, and four of them for its products);
+  and its mean error, which the sum over a lattice would carry, is within 2^-56 of
+  its terms' sizes (what rounding 4 dx^2 V's products down adds on average).
 
 The program prints each largest error over its bound."""
 import os
@@ -84,7 +86,7 @@ void run(const char* name, double base, double amp, double dx2, double q0, bool 
       site_force<NF, D, true, false>(G, NB, em, s, -(it & 1), F, en);
     }
     Q cpl = 0, eq = 0;
-    double cd = 0, mag = 0, slack = 0, grid = 0;
+    double cd = 0, mag = 0, slack = 0, grid = 0, pot = 0;
     for (int i = 1; i < NF; ++i) {
       cpl += (Q)q[i - 1] * g[i] * g[i];
       cd = std::fma(q[i - 1] * g[i], g[i], cd);
@@ -105,6 +107,7 @@ void run(const char* name, double base, double amp, double dx2, double q0, bool 
       const double model = std::fabs((double)((Q)dx2 * dv));
       size += model;
       slack += std::fabs(g[i]) * (std::ldexp((2 * D + 4) * mx, -57) + std::ldexp(model, -56));
+      pot += std::fabs(g[i]) * model;
       grid = std::fmax(grid, std::fabs(g[i]) * mx);
       if (size > 0) {
         const double bound =
@@ -121,8 +124,8 @@ void run(const char* name, double base, double amp, double dx2, double q0, bool 
     if (mag > 0) {
       const double e = (double)((Q)en - eq);
       energy = std::fmax(energy, std::fabs(e) / (std::ldexp(std::fabs((double)eq), -53) + slack +
-                                                 std::ldexp((NF + 1) * grid, -54)));
-      bias += e / std::ldexp(mag, -57);
+                                                 std::ldexp((NF + 1) * grid, -54) + std::ldexp((NF + 2) * pot, -55)));
+      bias += e / std::ldexp(mag, -56);
       ++terms;
     }
   }
