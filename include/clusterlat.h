@@ -271,7 +271,7 @@ int ce_load(ce_sim* sim, const char* path);
  * results (its items and their summation order do not depend on the mix). */
 typedef struct ce_batch ce_batch;
 
-/* sims: n handles; sweep_len: sites per item along the sweep axis (0 = 128);
+/* sims: n handles; sweep_len: sites per item along the sweep axis (0 = automatic);
  * ctas_per_sm: cap on the persistent kernel's resident CTAs per SM, 0..8
  * (0 = as many as fit); stream: cudaStream_t for the batch's work (NULL = its
  * own stream).

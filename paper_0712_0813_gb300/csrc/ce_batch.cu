@@ -74,13 +74,22 @@ struct BMember {
   DevScalars* slot;        // the lattice's two scalar slots
   int* status;
   unsigned int* done;      // items of this lattice completed in the running launch
-  double* partials;        // 2 doubles per item of this lattice
+  double* partials;        // one double per item of this lattice
   int dims, N, p0, first_item, n_items, update_scalars;   // 1D: n_items = blocks of the 1D launch
   int seg_log2;            // 3D: log2 of the lanes per row segment (5, 4 or 3: 1, 2 or 4 rows per warp)
   const CUtensorMap* tmaps;  // 3D: tensor maps of f, w (see kMapTypes), device memory; else null
   T inv_dx2, dt, q[3];
-  double ddt, kappa2, inv_S, half_inv_dx2;
+  double ddt, inv_ddt, kappa2;
+  SourceWeights source;
 };
+
+// A block's share of the member's 2 G + 3 V (valid in thread 0).
+__device__ __forceinline__ double member_source(const BMember<float>* m, float g2, float pot) {
+  return block_source(g2, 0.f, pot, 0.f, m->source);
+}
+__device__ __forceinline__ double member_source(const BMember<double>* m, double g2, double pot) {
+  return block_sum(fma(pot, (double)m->source.ratio + (double)m->source.ratio_lo, g2)) * m->source.weight;
+}
 
 struct BItem {
   int member;
@@ -470,12 +479,9 @@ __global__ void __launch_bounds__(kThreads, NF <= 2 ? 2 : 1) k_step_batched(cons
       break;
     }
     if (m->update_scalars) {
-      double g2, pot;
-      block_sum2_t<T>(g2loc, vloc, g2, pot);
+      const double share = member_source(m, g2loc, vloc);
       if (threadIdx.x == 0) {
-        const int k = itx - m->first_item;
-        m->partials[2 * k] = g2;
-        m->partials[2 * k + 1] = pot;
+        m->partials[itx - m->first_item] = share;
         __threadfence();
         s_last = atomicAdd(m->done, 1u) == (unsigned int)(m->n_items - 1);
       }
@@ -485,16 +491,12 @@ __global__ void __launch_bounds__(kThreads, NF <= 2 ? 2 : 1) k_step_batched(cons
         // (thread t takes items t, t + blockDim, ..., then a fixed tree, so the
         // order depends on the lattice's item count alone) and advances a
         __threadfence();
-        double G = 0.0, V = 0.0;
-        for (int j = threadIdx.x; j < m->n_items; j += blockDim.x) {
-          G += __ldcg(m->partials + 2 * j);
-          V += __ldcg(m->partials + 2 * j + 1);
-        }
-        block_sum2(G, V);
+        double sum = 0.0;
+        for (int j = threadIdx.x; j < m->n_items; j += blockDim.x) sum += __ldcg(m->partials + j);
+        sum = block_sum(sum);
         if (threadIdx.x == 0) {
           DevScalars out;
-          scale_factor_update(m->slot[in], out, G * m->half_inv_dx2 * m->inv_S, V * m->inv_S, m->ddt,
-                              m->kappa2, m->status);
+          scale_factor_update(scale_ahead(m->slot[in], m->ddt, m->kappa2), out, sum, m->inv_ddt, m->status);
           m->slot[in ^ 1] = out;
           *m->done = 0u;
         }
@@ -518,7 +520,7 @@ __global__ void __launch_bounds__(kThreads, NF <= 2 ? 2 : 1) k_step_batched(cons
 // lattice's n_items leave at once).  Per site the arithmetic is
 // step1d_group's (that of the single-lattice 1D kernel); a thread's sums stay
 // in T over its kG1d groups (16 sites in FP32, as in the other step kernels),
-// the block adds them with block_sum2_t into the lattice's partials, and the
+// the block adds them with member_source into the lattice's partials, and the
 // lattice's last block adds those in block order (thread t takes blocks t, t +
 // kThreads, ..., then a fixed tree) and advances its a, a', a''.  A lattice's
 // blocks and the order of its sums depend on its N alone, so its result does
@@ -555,27 +557,21 @@ __global__ void __launch_bounds__(kThreads) k_step_1d_members(const BMember<T>* 
   }
   if (!m->update_scalars) return;   // the same for every thread of the block
   __shared__ int s_last;
-  double g2, pot;
-  block_sum2_t<T>(g2loc, vloc, g2, pot);
+  const double share = member_source(m, g2loc, vloc);
   if (threadIdx.x == 0) {
-    m->partials[2 * blockIdx.x] = g2;
-    m->partials[2 * blockIdx.x + 1] = pot;
+    m->partials[blockIdx.x] = share;
     __threadfence();
     s_last = atomicAdd(m->done, 1u) == (unsigned int)(nb - 1);
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  double G = 0.0, V = 0.0;
-  for (int j = threadIdx.x; j < nb; j += kThreads) {
-    G += __ldcg(m->partials + 2 * j);
-    V += __ldcg(m->partials + 2 * j + 1);
-  }
-  block_sum2(G, V);
+  double sum = 0.0;
+  for (int j = threadIdx.x; j < nb; j += kThreads) sum += __ldcg(m->partials + j);
+  sum = block_sum(sum);
   if (threadIdx.x == 0) {
     DevScalars out;
-    scale_factor_update(m->slot[in], out, G * m->half_inv_dx2 * m->inv_S, V * m->inv_S, m->ddt, m->kappa2,
-                        m->status);
+    scale_factor_update(scale_ahead(m->slot[in], m->ddt, m->kappa2), out, sum, m->inv_ddt, m->status);
     m->slot[in ^ 1] = out;
     *m->done = 0u;
   }
@@ -593,7 +589,7 @@ struct ce_batch {
   void* d_items = nullptr;
   unsigned int* d_queue = nullptr;   // [0] head, [1] exit count
   unsigned int* d_done = nullptr;    // per member
-  double* d_partials = nullptr;      // 2 per item (and per block of a 1D member)
+  double* d_partials = nullptr;      // one per item (and per block of a 1D member)
   int* d_m1d = nullptr;              // indices of the 1D members
   int n1d = 0, bx1d = 0;             // 1D members; blocks of the largest one
   int n_units = 0;                   // items plus the 1D members' blocks
@@ -621,6 +617,13 @@ int bcuda(cudaError_t e, const char* what) {
 }
 
 constexpr int kBatchStages = 4;
+// Item length along the sweep axis where the caller gives none.  It may not depend on
+// the mix (a lattice's sums are those of its items).  us a step at 128 / 32 / 16 / 8:
+// FP32 mixes of 96 lattices 656 / 657 / 677 / 726, of 48 (3D sides to 160) 225 / 225 /
+// 232 / 246, of 18 183 / 116 / 122 / 127, of 6 (sides to 96) 99 / 42 / 36 / 35; FP64 of
+// 12 (sides to 128) 1295 / 1323 / 1075 / 1059.  Long items leave a small mix too few to
+// fill the CTAs, short ones pay for their two halo planes and the ring's start.
+constexpr int kItemLen32 = 32, kItemLen64 = 16;
 
 // One step: the persistent launch (2D/3D members) on the batch's stream and
 // the 1D launch on `st1d` (the side stream, or the batch's stream itself).
@@ -762,8 +765,8 @@ void build_tables(ce_batch* b, std::vector<ce::BMember<T>>& mem, std::vector<ce:
     for (int i = 0; i < 3; ++i) m.q[i] = (T)s->cfg.q[i];
     m.ddt = s->cfg.dt;
     m.kappa2 = s->kappa2;
-    m.inv_S = 1.0 / (double)s->S;
-    m.half_inv_dx2 = 0.5 / (s->dx * s->dx);
+    m.inv_ddt = 1.0 / s->cfg.dt;
+    m.source = ce::source_weights(s->dx, s->S);
     for (const Work& w : per[k]) items.push_back(w.it);
   }
 }
@@ -848,9 +851,9 @@ int upload_tables(ce_batch* b) {
     b->bx1d = std::max(b->bx1d, mem[k].n_items);
   }
   b->n_units = (int)slots;
-  cudaError_t e = cudaMalloc(&b->d_partials, sizeof(double) * 2 * std::max<int64_t>(1, slots));
+  cudaError_t e = cudaMalloc(&b->d_partials, sizeof(double) * std::max<int64_t>(1, slots));
   if (e != cudaSuccess) return bcuda(e, "ce_batch_create: partials");
-  for (auto& m : mem) m.partials = b->d_partials + 2 * (int64_t)m.first_item;
+  for (auto& m : mem) m.partials = b->d_partials + (int64_t)m.first_item;
   if (b->n1d > 0) {
     e = cudaMalloc(&b->d_m1d, sizeof(int) * m1d.size());
     if (e == cudaSuccess)
@@ -1020,7 +1023,7 @@ int ce_batch_create(ce_sim* const* sims, int n, int sweep_len, int ctas_per_sm, 
   b->prec = s0->prec;
   b->nf = s0->nf;
   b->device = s0->device;
-  b->sweep_len = sweep_len > 0 ? sweep_len : 128;
+  b->sweep_len = sweep_len > 0 ? sweep_len : (b->prec == CE_F32 ? kItemLen32 : kItemLen64);
   b->ctas_per_sm = ctas_per_sm;
   for (ce_sim* s : b->members) {
     e = cudaStreamSynchronize(s->stream);   // members' own queued work finishes first

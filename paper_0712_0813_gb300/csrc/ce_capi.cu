@@ -43,11 +43,23 @@ constexpr int kRowsMinN3 = 256;
 constexpr int kRowsMinN2 = 512;
 constexpr int kLinesMinN2 = 320;
 constexpr int kGraphSteps = 32;   // steps per captured CUDA graph (even: keeps the ping-pong parity)
+constexpr int kResidentCounterWords = 64;   // the counter has 256 bytes of its own
+constexpr int kResidentSteps = 4096;   // most steps of one resident launch
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz: bound of every device-side wait
 
 }  // namespace
 
 void ce::set_last_error(const std::string& msg) { g_err = msg; }
+
+// 2 G + 3 V = <(df)^2> / dx^2 + 3 <V> with G = <(df)^2> / (2 dx^2).
+ce::SourceWeights ce::source_weights(double dx, int64_t S) {
+  const double ratio = 3.0 * dx * dx;
+  SourceWeights w;
+  w.weight = 1.0 / (dx * dx * (double)S);
+  w.ratio = (float)ratio;
+  w.ratio_lo = (float)(ratio - (double)w.ratio);
+  return w;
+}
 
 
 namespace {
@@ -134,9 +146,9 @@ ce::StepArgs<T> make_step_args(const ce_sim* s, int in, bool half_kick) {
   a.dt_kick = half_kick ? (T)(0.5 * s->cfg.dt) : (T)s->cfg.dt;
   for (int i = 0; i < 3; ++i) a.q[i] = (T)s->cfg.q[i];
   a.dt = s->cfg.dt;
+  a.inv_dt = 1.0 / s->cfg.dt;
   a.kappa2 = s->kappa2;
-  a.inv_S = 1.0 / (double)s->S;
-  a.half_inv_dx2 = 0.5 / (s->dx * s->dx);
+  a.source = ce::source_weights(s->dx, s->S);
   a.update_scalars = (s->cfg.expansion && !half_kick) ? 1 : 0;
   a.in_slot = in;
   const bool stall = (s->cfg.flags & CE_FLAG_TEST_TMA_STALL) != 0;
@@ -165,6 +177,37 @@ cudaError_t launch_one_step(const ce_sim* s, int in, bool half_kick) {
 cudaError_t step_once(const ce_sim* s, int in, bool half_kick) {
   return s->prec == CE_F32 ? launch_one_step<float>(s, in, half_kick)
                            : launch_one_step<double>(s, in, half_kick);
+}
+
+// n steps of a small lattice by the resident kernel, from buffer set `in`.
+template <typename T>
+cudaError_t launch_resident_steps(ce_sim* s, int in, int n) {
+  ce::ResidentArgs<T> a{};
+  for (int b = 0; b < 2; ++b)
+    for (int i = 0; i < 4; ++i) {
+      a.f[b][i] = static_cast<T*>(s->f[b][i < s->nf ? i : 0]);
+      a.w[b][i] = static_cast<T*>(s->w[b][i < s->nf ? i : 0]);
+    }
+  a.plan = s->res;
+  a.N = (int)s->N;
+  a.in = in;
+  a.steps = n;
+  a.update_scalars = s->cfg.expansion ? 1 : 0;
+  a.dt = (T)s->cfg.dt;
+  a.inv_dx2 = (T)(1.0 / (s->dx * s->dx));
+  for (int i = 0; i < 3; ++i) a.q[i] = (T)s->cfg.q[i];
+  a.ddt = s->cfg.dt;
+  a.inv_ddt = 1.0 / s->cfg.dt;
+  a.kappa2 = s->kappa2;
+  a.source = ce::source_weights(s->dx, s->S);
+  if constexpr (sizeof(T) == 8) a.model = ce::fx_model(a.dt, a.inv_dx2, s->cfg.q);
+  a.slot = s->aux->slot;
+  a.counter = s->res_counter;
+  a.count0 = s->res_count;
+  a.shares = reinterpret_cast<double*>(s->res_counter + kResidentCounterWords);
+  a.status = &s->aux->status;
+  a.wait_cycles = kWaitCycles;
+  return ce::launch_resident(a, s->dims, s->nf, s->stream);
 }
 
 // Capture kGraphSteps consecutive step launches starting from buffer set
@@ -451,7 +494,7 @@ int ce_create(const ce_config* cfg, ce_sim** out) {
   }
   planes_blocks = std::max(planes_blocks, fx_blocks);
   int64_t nblk = std::max<int64_t>(std::max<int64_t>(s->generic_blocks, std::max(sweep_blocks, planes_blocks)), 1);
-  int64_t plen = std::max<int64_t>(2 * nblk, (int64_t)s->diag_blocks_max * 17);
+  int64_t plen = std::max<int64_t>(nblk, (int64_t)s->diag_blocks_max * 17);
   s->partials = static_cast<double*>(dalloc(s, (size_t)plen * 8));
   s->aux = static_cast<ce::DevAux*>(dalloc(s, sizeof(ce::DevAux)));
   s->chunk = std::min<int64_t>(S, kStagingChunk);
@@ -480,6 +523,23 @@ int ce_create(const ce_config* cfg, ce_sim** out) {
       cudaGetLastError();
       g_err.clear();
       s->kernel = CE_KERNEL_GENERIC;   // automatic choice: fall back to the generic kernel
+    }
+  }
+  if (cfg->kernel == CE_KERNEL_AUTO && !sweep_hinted && !(cfg->flags & CE_FLAG_TEST_TMA_STALL)) {
+    s->res = s->prec == CE_F32 ? ce::resident_plan_f32(s->dims, s->N, s->nf, s->device, s->sms)
+                               : ce::resident_plan_f64(s->dims, s->N, s->nf, s->device, s->sms);
+    if (s->res.blocks > 0) {
+      const size_t bytes = kResidentCounterWords * sizeof(unsigned) + (size_t)s->res.blocks * 2 * sizeof(double);
+      s->res_counter = static_cast<unsigned*>(dalloc(s, bytes));
+      if (!s->res_counter) {
+        ce_free(s);
+        return fail(CE_ENOMEM, "ce_create: device allocation of scratch failed");
+      }
+      e = cudaMemsetAsync(s->res_counter, 0, bytes, s->stream);
+      if (e != cudaSuccess) {
+        ce_free(s);
+        return cuda_fail(e, "ce_create: init");
+      }
     }
   }
   e = cudaMemsetAsync(s->aux, 0, sizeof(ce::DevAux), s->stream);
@@ -533,6 +593,10 @@ int ce_set_fields(ce_sim* s, const double* f, const double* v, int mode, const c
     if ((rc = upload_field(s, v + (int64_t)i * s->S, s->w[s->cur][i]))) return rc;
   }
   cudaError_t e = cudaMemsetAsync(&s->aux->status, 0, sizeof(int), s->stream);
+  if (e == cudaSuccess && s->res_counter) {   // a launch that timed out has left it short
+    e = cudaMemsetAsync(s->res_counter, 0, sizeof(unsigned), s->stream);
+    s->res_count = 0;
+  }
   if (e != cudaSuccess) return cuda_fail(e, "ce_set_fields");
   ce::DevAux host{};
   if (mode == CE_VEL_SYNC) {
@@ -575,6 +639,22 @@ int ce_step(ce_sim* s, int64_t n) {
   if (!s->have_state) return fail(CE_ESTATE, "ce_step: no fields set (call ce_set_fields first)");
   if (s->batch) return fail(CE_ESTATE, "ce_step: the handle is a member of a batch (use ce_batch_step)");
   if ((rc = select_device(s))) return rc;
+  if (s->res.blocks > 0 && n > 0) {
+    // a captured launch would be replayed with the count of this call: plain launches there
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s->stream, &cap);
+    if (e != cudaSuccess) return cuda_fail(e, "ce_step");
+    while (n > 0 && cap == cudaStreamCaptureStatusNone) {
+      const int m = (int)std::min<int64_t>(n, kResidentSteps);
+      e = s->prec == CE_F32 ? launch_resident_steps<float>(s, s->cur, m) : launch_resident_steps<double>(s, s->cur, m);
+      if (e != cudaSuccess) return cuda_fail(e, "ce_step: launch");
+      s->res_count += (uint32_t)m * (uint32_t)s->res.blocks;
+      s->cur ^= m & 1;
+      for (int k = 0; k < m; ++k) s->t = s->t + s->cfg.dt;
+      s->step += m;
+      n -= m;
+    }
+  }
   while (n >= kGraphSteps && s->graphs_ok) {
     cudaError_t e = ensure_graph(s, s->cur);
     if (e != cudaSuccess) {

@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kColThreads, MB) k_step_cols(const StepArgs<T>
     }
     if (k <= np - 2) stage(k, gB, gC3, gA, vC3, vA);
   }
-  if (p.update_scalars) finish_step_block(p, (double)g2acc + (double)g2loc, (double)vacc + (double)vloc);
+  if (p.update_scalars) finish_step_sums(p, g2acc, g2loc, vacc, vloc);
 }
 
 template <typename T, int NF>

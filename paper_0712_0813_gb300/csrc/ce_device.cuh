@@ -126,55 +126,84 @@ __device__ __forceinline__ int64_t grid_blocks() {
   return (int64_t)gridDim.x * gridDim.y * gridDim.z;
 }
 
-// Fixed-order block sum of two values; the result is valid in thread 0.
-__device__ __forceinline__ void block_sum2(double& a, double& b) {
-  __shared__ double sa[32], sb[32];
+// FP64 is scarce here: a warp instruction takes one of the SM's four FP64 pipes for
+// 64 cycles, whether one lane needs it or 32, and its result as long (measured: add,
+// multiply, FMA and conversion 64 each, division 554, square root 607).  So what
+// runs once per block or per step is written for few FP64 instructions: the end of
+// a block and of a launch below took ~6 us of a step, the launch gap ~2.
+
+// hi + lo += x: the addition's rounding error (Knuth's TwoSum, exact) joins lo.
+__device__ __forceinline__ void add_to(float& hi, float& lo, float x) {
+  const float s = hi + x;
+  const float b = s - hi;
+  lo += (hi - (s - b)) + (x - b);
+  hi = s;
+}
+
+// A sum kept as an unevaluated pair of floats (48 bits).
+struct FloatPair {
+  float hi, lo;
+};
+// Sum of the lanes' pairs (valid in lane 0; lanes of `width` only).
+template <int WIDTH>
+__device__ __forceinline__ void warp_sum_pair(FloatPair& x) {
+#pragma unroll
+  for (int o = WIDTH / 2; o > 0; o >>= 1) {
+    x.lo += __shfl_down_sync(0xffffffffu, x.lo, o);
+    add_to(x.hi, x.lo, __shfl_down_sync(0xffffffffu, x.hi, o));
+  }
+}
+
+// A block's share of 2 G + 3 V from its threads' two-level FP32 sums g0 + g1 and
+// v0 + v1 (fixed order, valid in thread 0).  The sums are combined and added as float
+// pairs (the per-thread sums' own rounding stays what limits them): three FP64
+// instructions a block; sums that would leave FP32's range take FP64 throughout.
+__device__ __forceinline__ double block_source(float g0, float g1, float v0, float v1, const SourceWeights& k) {
+  __shared__ float2 part[32];
+  __shared__ double wide[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nwarps = (blockDim.x + 31) >> 5;
+  FloatPair t{g0, 0.f}, v{v0, 0.f};
+  add_to(t.hi, t.lo, g1);
+  add_to(v.hi, v.lo, v1);
+  const float p = __fmul_rn(k.ratio, v.hi);
+  t.lo += fmaf(k.ratio, v.hi, -p) + fmaf(k.ratio_lo, v.hi, k.ratio * v.lo);
+  add_to(t.hi, t.lo, p);
+  const bool fits = fabsf(t.hi) < 1e32f;
+  warp_sum_pair<32>(t);
+  if (lane == 0) part[warp] = make_float2(t.hi, t.lo);
+  if (__syncthreads_or(!fits)) {
+    const double q = warp_sum(fma((double)v0 + (double)v1, (double)k.ratio + (double)k.ratio_lo, (double)g0 + (double)g1));
+    if (lane == 0) wide[warp] = q;
+    __syncthreads();
+    double sum = 0.0;
+    if (threadIdx.x == 0)
+      for (int w = 0; w < nwarps; ++w) sum += wide[w];
+    return sum * k.weight;
+  }
+  double q = 0.0;
+  if (warp == 0) {
+    const float2 x = lane < nwarps ? part[lane] : make_float2(0.f, 0.f);
+    FloatPair s{x.x, x.y};
+    warp_sum_pair<32>(s);
+    if (lane == 0) q = ((double)s.hi + (double)s.lo) * k.weight;
+  }
+  return q;
+}
+
+// Sum over the block of one FP64 value, fixed order, valid in thread 0.
+__device__ __forceinline__ double block_sum(double a) {
+  __shared__ double part[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = (blockDim.x + 31) >> 5;
   a = warp_sum(a);
-  b = warp_sum(b);
-  if (lane == 0) { sa[warp] = a; sb[warp] = b; }
+  if (lane == 0) part[warp] = a;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double x = 0.0, y = 0.0;
-    for (int w = 0; w < nwarps; ++w) { x += sa[w]; y += sb[w]; }
-    a = x;
-    b = y;
+  if (warp == 0) {
+    a = lane < nwarps ? part[lane] : 0.0;
+    for (int o = nwarps > 16 ? 16 : (nwarps > 8 ? 8 : 4); o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
   }
-  __syncthreads();
-}
-
-// Block sum of two per-thread values of the storage type T: a fixed tree of
-// shuffles inside each warp in T, then the warps' sums added in FP64, in warp
-// order, by thread 0.  For T = float this keeps the FP64 work of a block at
-// two additions per warp (GB300's FP64 pipe is narrow: a warp-wide FP64
-// instruction occupies it for 16 cycles); the tree over 32 values adds at most
-// ~5 rounding steps of 2^-24 to each warp's sum.  Result valid in thread 0.
-template <typename T>
-__device__ __forceinline__ void block_sum2_t(T a, T b, double& oa, double& ob) {
-  __shared__ double sa[32], sb[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarps = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
-  }
-  if (lane == 0) {
-    sa[warp] = (double)a;
-    sb[warp] = (double)b;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double x = 0.0, y = 0.0;
-    for (int w = 0; w < nwarps; ++w) {
-      x += sa[w];
-      y += sb[w];
-    }
-    oa = x;
-    ob = y;
-  }
-  __syncthreads();
+  return a;
 }
 
 // Scale-factor update of reading c-4, done once per step by one thread:
@@ -183,39 +212,61 @@ __device__ __forceinline__ void block_sum2_t(T a, T b, double& oa, double& ob) {
 //   u = a'_{n+3/2} + a'_{n+1/2} = 2 C / (1 + sqrt(1 + dt C / a_{n+1}))
 // (closed form of the implicit midpoint a'_new - a'_old = dt (-(u/2)^2/a + Q)),
 //   a''_{n+1} = (u - 2 a'_{n+1/2}) / dt,  a'_{n+3/2} = u - a'_{n+1/2}.
-__device__ __forceinline__ void scale_factor_update(const DevScalars& in, DevScalars& out, double G,
-                                                    double V, double dt, double kappa2, int* status) {
-  const double a = in.a + dt * in.ap;
-  const double Q = kappa2 * (2.0 * G + 3.0 * V) / a;
-  const double C = 2.0 * in.ap + dt * Q;
-  const double disc = 1.0 + dt * C / a;
-  if (!(disc >= 0.0) || !isfinite(G) || !isfinite(V)) atomicCAS(status, CE_OK, CE_ENONFINITE);
-  const double u = 2.0 * C / (1.0 + sqrt(disc));
-  const double app = (u - 2.0 * in.ap) / dt;
-  out.a = a;
-  out.ap = u - in.ap;
+// In two parts: what does not need the sums (scale_ahead) can run before they are
+// there.  y = u / C solves (e/4) y^2 + y = 1 with e = dt C / a: for small e two
+// Newton steps in FP64 with FP32's slope, from FP32's root (errors 1e-7, 1e-14, 0),
+// are six instructions where the square root and the division take eighteen.
+struct ScaleAhead {
+  double a, ap, ap2, ia, dia, k1, e1;
+};
+__device__ __forceinline__ ScaleAhead scale_ahead(const DevScalars& in, double dt, double kappa2) {
+  ScaleAhead s;
+  s.a = fma(dt, in.ap, in.a);
+  s.ap = in.ap;
+  s.ap2 = in.ap + in.ap;
+  s.ia = 1.0 / s.a;
+  s.dia = dt * s.ia;
+  s.k1 = kappa2 * s.dia;
+  s.e1 = 0.25 * s.dia;
+  return s;
+}
+// source: 2 G + 3 V.
+__device__ __forceinline__ void scale_factor_update(const ScaleAhead& s, DevScalars& out, double source, double inv_dt,
+                                                    int* status) {
+  const double C = fma(s.k1, source, s.ap2);
+  const double e4 = s.e1 * C;
+  const float e = 4.f * (float)e4;
+  double y;
+  if (fabsf(e) < 0.25f) {
+    const float yf = 2.f / (1.f + sqrtf(1.f + e));
+    const double slope = (double)(1.f / (1.f + 0.5f * e * yf));
+    y = (double)yf;
+    y = fma(fma(-(e4 * y), y, 1.0 - y), slope, y);
+    y = fma(fma(-(e4 * y), y, 1.0 - y), slope, y);
+  } else {   // also where something is not finite
+    const double disc = fma(4.0, e4, 1.0);
+    if (!(disc >= 0.0) || !isfinite(source)) atomicCAS(status, CE_OK, CE_ENONFINITE);
+    y = 2.0 / (1.0 + sqrt(disc));
+  }
+  const double u = C * y;
+  const double app = (u - s.ap2) * inv_dt;
+  out.c = app * s.dia;
   out.app = app;
-  out.s = app / a;
-  out.c = dt * out.s;
-  out.G = G;
-  out.V = V;
-  out.pad = 0.0;
+  out.s = app * s.ia;
+  out.a = s.a;
+  out.ap = u - s.ap;
 }
 
-// End of a step launch: reduce this block's partial sums of
-//   sum (f(x+e_d) - f(x))^2   and   sum V(f(x))
-// in a fixed order, publish them, and let the last block to finish combine all
-// blocks' partials (fixed order over block index) and advance a, a', a''.
-// No block ever waits for another: the last arriving block does the work.
+// End of a step launch: publish this block's share of 2 G + 3 V (in thread 0), and
+// let the last block to finish combine all blocks' shares (fixed order over block
+// index) and advance a, a', a''.  No block ever waits for another: the last
+// arriving block does the work.
 template <typename T>
-__device__ __forceinline__ void finish_step_block(const StepArgs<T>& p, double grad2, double pot) {
+__device__ __forceinline__ void finish_step(const StepArgs<T>& p, double share) {
   __shared__ int am_last;
-  block_sum2(grad2, pot);
   const int64_t nb = grid_blocks();
   if (threadIdx.x == 0) {
-    const int64_t b = linear_block_id();
-    p.partials[2 * b] = grad2;
-    p.partials[2 * b + 1] = pot;
+    p.partials[linear_block_id()] = share;
     __threadfence();
     const unsigned int prev = atomicAdd(p.counter, 1u);
     am_last = (prev == (unsigned int)(nb - 1));
@@ -223,19 +274,27 @@ __device__ __forceinline__ void finish_step_block(const StepArgs<T>& p, double g
   __syncthreads();
   if (!am_last) return;
   __threadfence();
-  double g = 0.0, v = 0.0;
-  for (int64_t j = threadIdx.x; j < nb; j += blockDim.x) {
-    g += __ldcg(p.partials + 2 * j);
-    v += __ldcg(p.partials + 2 * j + 1);
-  }
-  block_sum2(g, v);
+  ScaleAhead ahead;
+  if (threadIdx.x == 0) ahead = scale_ahead(*p.sc_in, p.dt, p.kappa2);
+  double sum = 0.0;
+  for (int64_t j = threadIdx.x; j < nb; j += blockDim.x) sum += __ldcg(p.partials + j);
+  sum = block_sum(sum);
   if (threadIdx.x == 0) {
     DevScalars out;
-    scale_factor_update(*p.sc_in, out, g * p.half_inv_dx2 * p.inv_S, v * p.inv_S, p.dt, p.kappa2,
-                        p.status);
+    scale_factor_update(ahead, out, sum, p.inv_dt, p.status);
     *p.sc_out = out;
     *p.counter = 0u;
   }
+}
+
+// The same from the threads' FP32 sums of (df)^2 and V, in two levels each.
+__device__ __forceinline__ void finish_step_sums(const StepArgs<float>& p, float g0, float g1, float v0, float v1) {
+  finish_step(p, block_source(g0, g1, v0, v1, p.source));
+}
+// And from FP64 sums.
+__device__ __forceinline__ void finish_step_sums(const StepArgs<double>& p, double g0, double g1, double v0, double v1) {
+  const double ratio = (double)p.source.ratio + (double)p.source.ratio_lo;
+  finish_step(p, block_sum(fma(v0 + v1, ratio, g0 + g1)) * p.source.weight);
 }
 
 }  // namespace ce

@@ -120,14 +120,6 @@ __device__ __forceinline__ void diag_site(const DiagScalars<T>& k, int raw_u, co
   }
 }
 
-// hi + lo += x: the addition's rounding error (Knuth's TwoSum, exact) joins lo.
-__device__ __forceinline__ void add_to(float& hi, float& lo, float x) {
-  const float s = hi + x;
-  const float b = s - hi;
-  lo += (hi - (s - b)) + (x - b);
-  hi = s;
-}
-
 // A thread's running sums: FP64, or float pairs.  Partials of 2^100 and above,
 // infinities and NaN would leave the pairs' range: they go to the block's FP64
 // sums `big` in shared memory.

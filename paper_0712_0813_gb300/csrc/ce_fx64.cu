@@ -23,7 +23,7 @@
 #include <cstdint>
 
 #include "ce_device.cuh"
-#include "ce_fx.cuh"
+#include "ce_fx_force.cuh"
 #include "ce_internal.h"
 #include "ce_plan.h"
 #include "ce_tma.cuh"
@@ -37,56 +37,6 @@ constexpr int kFxWarps = 4;
 constexpr int kFxThreads = 32 * kFxWarps;
 constexpr int kStrip = 30;   // sites a warp updates along x
 
-// The force of a site one of whose stencil values is infinite or NaN, in FP64.
-template <int NF, int DIMS>
-__device__ __noinline__ void force_fp64(const double* g, const double* nb, double dx2, const double* q, double* force,
-                                        double* energy) {
-  double gs[NF], dv[NF], vs, e = 0.0;
-  for (int i = 0; i < NF; ++i) gs[i] = g[i];
-  const double qs[3] = {q[0], q[1], q[2]};
-  model_dv<double, NF>(gs, qs, dv, vs);
-  for (int i = 0; i < NF; ++i) {
-    double raw = -2.0 * DIMS * gs[i];
-    for (int j = 0; j < 2 * DIMS; ++j) raw += nb[i * 2 * DIMS + j];
-    force[i] = fma(-dx2, dv[i], raw);
-    e += gs[i] * fma(-0.75 * dx2, dv[i], raw);
-  }
-  *energy = e;
-}
-
-// The site's force by the form its values allow.
-template <int NF, int DIMS, bool SUMS>
-__device__ __forceinline__ void force_of(const Fx (&g)[NF], const Fx (&nb)[NF][2 * DIMS], const fx::FxModel& k,
-                                         const StepArgs<double>& p, double (&force)[NF], double& energy) {
-  const int flip = -(int)(threadIdx.x & 1u);
-  int em[NF];
-  fx::stencil_exponents<NF, DIMS>(g, nb, em);
-  fx::SiteModel<NF> s;
-  fx::site_model<NF, SUMS>(g, k, s);
-  if (fx::fast_site<NF>(em, s)) {
-    fx::site_force<NF, DIMS, SUMS, true>(g, nb, em, s, flip, force, energy);
-    return;
-  }
-  int most = em[0];
-#pragma unroll
-  for (int i = 1; i < NF; ++i) most = max(most, em[i]);
-  if (most < fx::kNonFinite) {
-    fx::site_force<NF, DIMS, SUMS, false>(g, nb, em, s, flip, force, energy);
-    return;
-  }
-  double gd[NF], nd[NF * 2 * DIMS], fd[NF], qd[3] = {p.q[0], p.q[1], p.q[2]}, ed;
-#pragma unroll
-  for (int i = 0; i < NF; ++i) {
-    gd[i] = fx::to_double(g[i]);
-#pragma unroll
-    for (int j = 0; j < 2 * DIMS; ++j) nd[i * 2 * DIMS + j] = fx::to_double(nb[i][j]);
-  }
-  force_fp64<NF, DIMS>(gd, nd, 1.0 / p.inv_dx2, qd, fd, &ed);
-#pragma unroll
-  for (int i = 0; i < NF; ++i) force[i] = fd[i];
-  energy = ed;
-}
-
 __device__ __forceinline__ Fx shfl_up(const Fx& x) {
   return Fx{__shfl_up_sync(0xffffffffu, x.m, 1), __shfl_up_sync(0xffffffffu, x.e, 1)};
 }
@@ -94,9 +44,10 @@ __device__ __forceinline__ Fx shfl_down(const Fx& x) {
   return Fx{__shfl_down_sync(0xffffffffu, x.m, 1), __shfl_down_sync(0xffffffffu, x.e, 1)};
 }
 
-// End of a step: the block's energy sum, and in the launch's last block a, a', a''
-// (2 G + 3 V = -dx^-2 <energy>, passed on as G with V = 0).
-__device__ __forceinline__ void finish(const StepArgs<double>& p, double energy) { finish_step_block(p, -energy, 0.0); }
+// End of a step from the threads' energy terms: 2 G + 3 V = -dx^-2 <energy>.
+__device__ __forceinline__ void finish(const StepArgs<double>& p, double energy) {
+  finish_step(p, block_sum(energy) * -p.source.weight);
+}
 
 // ---- 3D ---------------------------------------------------------------------
 // A block owns 30 x-sites by RB rows and sweeps a chunk of z: RB + 2 warps, one
@@ -145,6 +96,7 @@ __global__ void __launch_bounds__(32 * (RB + 2), FxRows<NF>::blocks)
   int zq = z0 == 0 ? N - 1 : z0 - 1;
   int64_t oq = zq * NN + here, oN = oq, oC = oq;
   const double c = p.sc_in->c, dd = p.dt_drift, kk = p.dt_kick * p.inv_dx2;
+  const double q[3] = {p.q[0], p.q[1], p.q[2]};
   double lf[NF], lw[NF];                         // loads under way: the next plane to form
   const auto issue = [&]() {
     const int64_t o = oq;
@@ -221,7 +173,7 @@ __global__ void __launch_bounds__(32 * (RB + 2), FxRows<NF>::blocks)
       }
       if (site) {
         double force[NF], energy;
-        force_of<NF, 3, SUMS>(gC, nb, k, p, force, energy);
+        fx::force_of<NF, 3, SUMS>(gC, nb, k, p.inv_dx2, q, force, energy);
         if constexpr (SUMS) acc += energy;
 #pragma unroll
         for (int i = 0; i < NF; ++i) p.w_out[i][oC] = fma(kk, force[i], vC[i]);
@@ -262,6 +214,7 @@ __global__ void __launch_bounds__(kFxThreads, 3) k_step_fx2(const StepArgs<doubl
       return y * N + xs;
     };
     const double c = p.sc_in->c, dd = p.dt_drift, kk = p.dt_kick * p.inv_dx2;
+    const double q[3] = {p.q[0], p.q[1], p.q[2]};
     double lf[DL][NF], lw[DL][NF];
     const auto issue = [&](int j, int slot) {
       const int64_t o = row_off(j);
@@ -311,7 +264,7 @@ __global__ void __launch_bounds__(kFxThreads, 3) k_step_fx2(const StepArgs<doubl
         }
         if (site) {
           double force[NF], energy;
-          force_of<NF, 2, SUMS>(gc, nb, k, p, force, energy);
+          fx::force_of<NF, 2, SUMS>(gc, nb, k, p.inv_dx2, q, force, energy);
           if constexpr (SUMS) acc += energy;
           const int64_t o = row_off(j - 1);
 #pragma unroll
@@ -329,6 +282,7 @@ __global__ void __launch_bounds__(kFxThreads) k_step_fx1(const StepArgs<double> 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t N = p.N, stride = (int64_t)gridDim.x * kFxWarps;
   const double c = p.sc_in->c, dd = p.dt_drift, kk = p.dt_kick * p.inv_dx2;
+  const double q[3] = {p.q[0], p.q[1], p.q[2]};
   double acc = 0.0;
   const auto column = [&](int64_t strip) -> int64_t {
     const int64_t x0 = strip * kStrip, nx = min((int64_t)kStrip, N - x0);
@@ -366,7 +320,7 @@ __global__ void __launch_bounds__(kFxThreads) k_step_fx1(const StepArgs<double> 
     }
     if (site) {
       double force[NF], energy;
-      force_of<NF, 1, SUMS>(g, nb, k, p, force, energy);
+      fx::force_of<NF, 1, SUMS>(g, nb, k, p.inv_dx2, q, force, energy);
       if constexpr (SUMS) acc += energy;
 #pragma unroll
       for (int i = 0; i < NF; ++i) p.w_out[i][x] = fma(kk, force[i], v[i]);
@@ -391,17 +345,21 @@ fx::FxConst constant(long double x) {
 // inside the force is dt / kk to 64 bits: the model force then enters with dt
 // itself (with both constants rounded to FP64 the potential of the oscillating mean
 // field was off by 2e-14 after 1000 steps, 3e-15 with dt).
-fx::FxModel model_constants(const StepArgs<double>& a) {
+}  // namespace
+
+fx::FxModel fx_model(double dt_kick, double inv_dx2, const double* q) {
   fx::FxModel k;
-  const volatile double kk = a.dt_kick * a.inv_dx2;   // the kernels' own product
-  const long double dx2 = (long double)a.dt_kick / (long double)kk;
+  const volatile double kk = dt_kick * inv_dx2;   // the kernels' own product
+  const long double dx2 = (long double)dt_kick / (long double)kk;
   k.dx2 = constant(dx2);
   for (int i = 0; i < 3; ++i) {
-    k.q[i] = constant(a.q[i]);
-    k.qdx2[i] = constant((long double)a.q[i] * dx2);
+    k.q[i] = constant(q[i]);
+    k.qdx2[i] = constant((long double)q[i] * dx2);
   }
   return k;
 }
+
+namespace {
 
 template <int NF, bool SUMS>
 const void* kernel_of(int dims) {
@@ -423,7 +381,7 @@ const void* kernel(int dims, int nf, bool sums) {
 
 template <int NF, bool SUMS>
 void launch(const StepArgs<double>& a, const FxPlan& pl, cudaStream_t st) {
-  const fx::FxModel k = model_constants(a);
+  const fx::FxModel k = fx_model(a.dt_kick, a.inv_dx2, a.q);
   const dim3 grid(pl.gx, pl.gy);
   if (a.dims == 3)
     k_step_fx3<NF, FxRows<NF>::value, SUMS><<<grid, 32 * (FxRows<NF>::value + 2), 0, st>>>(a, k, pl.nstrips, pl.len);

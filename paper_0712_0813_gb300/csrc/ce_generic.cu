@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kGenericThreads) k_step_generic(const StepArgs
       since_flush = 0;
     }
   }
-  if (p.update_scalars) finish_step_block(p, (double)g2acc + (double)g2loc, (double)vacc + (double)vloc);
+  if (p.update_scalars) finish_step_sums(p, g2acc, g2loc, vacc, vloc);
 }
 
 // One site s of a 1D lattice with the arithmetic of step1d_group (the sites
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kGenericThreads) k_step_1d(const StepArgs<T> p
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1)
     for (int64_t s = groups * VX; s < N; ++s)
       step1d_site<T, NF>(p.f_in, p.w_in, p.f_out, p.w_out, N, s, c, dd, kk, idx2, q, g2loc, vloc);
-  if (p.update_scalars) finish_step_block(p, (double)g2acc + (double)g2loc, (double)vacc + (double)vloc);
+  if (p.update_scalars) finish_step_sums(p, g2acc, g2loc, vacc, vloc);
 }
 
 template <typename T, int NF>
@@ -359,14 +359,13 @@ __global__ void k_init_scalars(DevAux* aux, int cur, int expansion, double dt, d
     app0 = (-ap0 * ap0 + kappa2 * (2.0 * G + 3.0 * V)) / a;
   }
   DevScalars s0;
-  s0.a = a; s0.ap = ap0; s0.app = 0.0; s0.s = 0.0; s0.c = ap0 / a; s0.G = G; s0.V = V; s0.pad = 0.0;
+  s0.a = a; s0.ap = ap0; s0.app = 0.0; s0.s = 0.0; s0.c = ap0 / a;
   DevScalars s1;
   s1.a = a;
   s1.ap = ap0 + 0.5 * dt * app0;
   s1.app = app0;
   s1.s = app0 / a;
   s1.c = 0.5 * dt * s1.s;
-  s1.G = G; s1.V = V; s1.pad = 0.0;
   aux->slot[cur] = s0;
   aux->slot[cur ^ 1] = s1;
 }

@@ -8,6 +8,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "ce_fx.cuh"
 #include "clusterlat.h"
 
 namespace ce {
@@ -26,9 +27,6 @@ struct DevScalars {
   double app;  // a''(t_n)
   double s;    // a''(t_n) / a(t_n)
   double c;    // coefficient of f in the velocity reconstruction above
-  double G;    // mean gradient energy of f(t_n) (when computed by a step)
-  double V;    // mean potential energy of f(t_n)
-  double pad;
 };
 
 constexpr int kResultLen = 64;
@@ -57,6 +55,15 @@ struct DevAux {
   double result[kResultLen];
 };
 
+// How a block's sums enter the source 2 G + 3 V of the scale factor: weight times
+// (sum of (df)^2 + ratio times sum of V), the ratio 3 dx^2 as a float pair.
+struct SourceWeights {
+  double weight;
+  float ratio, ratio_lo;
+};
+
+SourceWeights source_weights(double dx, int64_t S);
+
 // Arguments of one step launch.  T is the storage/arithmetic type of fields
 // and velocities; the global sums and scalars are always double.
 template <typename T>
@@ -73,17 +80,16 @@ struct StepArgs {
   T dt_drift;      // dt for a step, 0 for the start-up half kick
   T dt_kick;       // dt for a step, dt/2 for the start-up half kick
   T q[3];
-  double dt;
+  double dt, inv_dt;
   double kappa2;
-  double inv_S;
-  double half_inv_dx2;
+  SourceWeights source;
   int update_scalars;   // 1: reduce G, V and advance a, a', a'' in the last block
   int in_slot;          // which ping-pong buffer set is the input (selects TMA maps)
   long long wait_cycles;      // bound of every mbarrier wait (SM clock cycles)
   unsigned int missing_tx;    // test-only: bytes announced per plane that never arrive
   const DevScalars* sc_in;
   DevScalars* sc_out;
-  double* partials;     // >= 2 * number of blocks
+  double* partials;     // one per block
   unsigned int* counter;
   int* status;
 };
@@ -172,6 +178,34 @@ struct FxPlan {
 };
 FxPlan fx_plan(int dims, int64_t N, int nf, int sms);
 cudaError_t launch_step_fx(const StepArgs<double>& a, const FxPlan& plan, cudaStream_t st);
+fx::FxModel fx_model(double dt_kick, double inv_dx2, const double* q);
+// Many steps of a small lattice in one cooperative launch (ce_resident.cuh):
+// bricks of bx x by x bz sites, nx x ny x nz of them, one block each; blocks == 0
+// where the lattice does not take that kernel.
+struct ResidentPlan {
+  int bx, by, bz, nx, ny, nz, blocks, threads, smem;
+};
+template <typename T>
+struct ResidentArgs {
+  T* f[2][4];
+  T* w[2][4];
+  ResidentPlan plan;
+  int N, in, steps, update_scalars;
+  T dt, inv_dx2, q[3];
+  double ddt, inv_ddt, kappa2;
+  SourceWeights source;
+  fx::FxModel model;                        // FP64
+  DevScalars* slot;
+  double* shares;                           // 2 x blocks
+  unsigned* counter;                        // blocks that have published, over all steps so far (mod 2^32)
+  unsigned count0;                          // its value before the launch
+  int* status;
+  long long wait_cycles;
+};
+ResidentPlan resident_plan_f32(int dims, int64_t N, int nf, int device, int sms);
+ResidentPlan resident_plan_f64(int dims, int64_t N, int nf, int device, int sms);
+cudaError_t launch_resident(const ResidentArgs<float>& a, int dims, int nf, cudaStream_t st);
+cudaError_t launch_resident(const ResidentArgs<double>& a, int dims, int nf, cudaStream_t st);
 namespace sweep {
 cudaError_t launch_f32(int variant, const StepArgs<float>& a, const SweepMaps& m, dim3 grid, size_t smem,
                        cudaStream_t st);
@@ -215,6 +249,9 @@ struct ce_sim {
   ce::ColsPlan cols{};
   ce::LinesPlan lines{};
   ce::FxPlan fx{};             // FP64 handles on CE_KERNEL_GENERIC
+  ce::ResidentPlan res{};      // small lattices on the automatic kernel choice
+  unsigned* res_counter = nullptr;   // and, 256 bytes on, 2 x blocks shares
+  uint32_t res_count = 0;            // the counter's value after the launches so far
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // kGraphSteps steps starting from buffer set 0 / 1
   bool graphs_ok = true;
   int64_t bytes = 0;

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kLineThreads) k_step_lines(const StepArgs<T> p
       }
     }
   }
-  if (p.update_scalars) finish_step_block(p, (double)g2acc + (double)g2loc, (double)vacc + (double)vloc);
+  if (p.update_scalars) finish_step_sums(p, g2acc, g2loc, vacc, vloc);
 }
 
 template <typename T, int NF>

@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(32 * (TY + 1), (min_blocks<T, NF, TY, NST>()))
     return true;
   };
 
-  double grad2 = 0.0, pot = 0.0;
+  T grad2 = T(0), pot = T(0);   // the thread's sums
   int issued = 0;
   if (producer) {
     // ---------------- producer warp: one lane streams planes into the ring
@@ -378,8 +378,8 @@ __global__ void __launch_bounds__(32 * (TY + 1), (min_blocks<T, NF, TY, NST>()))
       }
     }
     if (lane == 0) atomicMin(&s_min_waited, waited);
-    grad2 = (double)g2loc;
-    pot = (double)vloc;
+    grad2 = g2loc;
+    pot = vloc;
   }
   __syncthreads();
   if (s_abort) {
@@ -393,10 +393,10 @@ __global__ void __launch_bounds__(32 * (TY + 1), (min_blocks<T, NF, TY, NST>()))
       }
     }
     __syncthreads();
-    grad2 = 0.0;
-    pot = 0.0;
+    grad2 = T(0);
+    pot = T(0);
   }
-  if (p.update_scalars) finish_step_block(p, grad2, pot);
+  if (p.update_scalars) finish_step_sums(p, grad2, T(0), pot, T(0));
 }
 
 
