@@ -53,10 +53,9 @@ __global__ void k_sample(SamplePtrs<T> p, int nf, const ce::DevScalars* sc, cons
 }
 
 constexpr int kBinThreads = 256;
-constexpr int kBinBlocks = 608;
-
-// Signed integer mode of index i along an axis of length N.
-__device__ __forceinline__ int64_t mode(int64_t i, int64_t N) { return i <= N / 2 ? i : i - N; }
+constexpr int kBinChunks = 16;      // most blocks a bin is shared out to (k_bin_spectrum)
+constexpr int kBinParts = 608;      // most partial histograms
+constexpr int kRowsSmem = 200 * 1024;   // shared memory of k_bin_rows per SM
 
 // Half-spectrum layout of a real-to-complex transform: the last (x) axis holds
 // N/2 + 1 modes.  Every stored mode except kx = 0 and the Nyquist kx = N/2
@@ -70,55 +69,273 @@ __global__ void k_shifted_copy(const T* __restrict__ f, T* __restrict__ out, int
     out[k] = f[k] - shift;
 }
 
-template <typename C, typename T>
+// floor(sqrt(x)) for 0 <= x < 2^34.
+__device__ __forceinline__ int isqrt(int64_t x) {
+  int s = (int)sqrtf((float)x);
+  while ((int64_t)s * s > x) --s;
+  while ((int64_t)(s + 1) * (s + 1) <= x) ++s;
+  return s;
+}
+
+// The same for 0 <= x < 2^24, exact in a float.
+__device__ __forceinline__ int isqrt(int x) {
+  int s;
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"((float)x));   // within one of the root
+  s = (int)r;
+  s -= s * s > x;
+  s += (s + 1) * (s + 1) <= x;
+  return s;
+}
+
+// w |F|^2 added to a thread's sum: FP64, or for FP32 spectra float pairs (48 bits,
+// the squares with their FMA residuals); values whose squares would leave FP32's
+// range, infinities and NaN take FP64.
+struct PowerSum {
+  double wide = 0.0;
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(double re, double im, double w) { wide += w * (re * re + im * im); }
+  __device__ __forceinline__ void add(float re, float im, float w) {
+    const float big = fmaxf(fabsf(re), fabsf(im)), small = fminf(fabsf(re), fabsf(im));
+    if (big < 0x1p50f && (small >= 0x1p-50f || small == 0.f) && (big >= 0x1p-50f || big == 0.f)) {
+      const float p = re * re, q = im * im;
+      ce::add_to(hi, lo, w * p);
+      ce::add_to(hi, lo, w * q);
+      lo += w * (fmaf(re, re, -p) + fmaf(im, im, -q));
+    } else {
+      add((double)re, (double)im, (double)w);
+    }
+  }
+  __device__ __forceinline__ double total() const { return wide + ((double)hi + (double)lo); }
+};
+
+// One bin (blockIdx.x) of the spectrum over a share (blockIdx.y) of the rows along x.
+// A mode n is in bin b when floor(|n| + 1/2) = b, for integers b^2 - b < n^2 <= b^2 + b
+// (bin 0: n = 0), so of the row at (ny, nz) it holds one run of nx, found from two
+// square roots.  Threads take rows, so no bin is shared between threads and nothing is
+// added atomically (a histogram in shared memory, with a 64-bit division chain, an FP64
+// square root and two FP64 compare-and-swap loops a mode, took most of 760 us at 256^3).
+// Bounded by the sectors a run touches (L2).
+// I: int where every n^2 is below 2^24, else int64_t.
+template <typename C, typename T, typename I>
 __global__ void __launch_bounds__(kBinThreads) k_bin_spectrum(const C* __restrict__ F, const T* __restrict__ f,
-                                                               int64_t N, int dims, int nbins,
+                                                               int64_t N64, int dims, int nbins,
                                                                double* __restrict__ part_p,
                                                                double* __restrict__ part_n) {
-  extern __shared__ double sh[];
-  double* hp = sh;
-  double* hn = sh + nbins;
-  for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
-    hp[b] = 0.0;
-    hn[b] = 0.0;
-  }
-  __syncthreads();
-  const int64_t nx = N / 2 + 1;
-  int64_t total = nx;
-  for (int d = 1; d < dims; ++d) total *= N;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t ix = k % nx;
-    int64_t rest = k / nx;
-    double n2 = (double)ix * (double)ix;
-    for (int d = 1; d < dims; ++d) {
-      const int64_t m = mode(rest % N, N);
-      rest /= N;
-      n2 += (double)m * (double)m;
+  __shared__ double sp[kBinThreads / 32];
+  __shared__ unsigned long long sn[kBinThreads / 32];
+  const I N = (I)N64, half = N / 2, b = (I)blockIdx.x;
+  const int64_t nx = half + 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const I first = b == 0 ? 0 : b * b - b + 1, last = b * b + b;   // n^2 in the bin
+  const I kmin = -min(b, (N - 1) / 2), kmax = min(b, half);       // ny, nz that can be in it
+  const I zmin = dims == 3 ? kmin : 0, zmax = dims == 3 ? kmax : 0;
+  const I ymin = dims >= 2 ? kmin : 0, ymax = dims >= 2 ? kmax : 0;
+  // 3D: warps take nz, lanes ny; else every thread takes rows ny
+  const I z_at = dims == 3 ? (I)blockIdx.y * (kBinThreads / 32) + warp : 0;
+  const I z_by = dims == 3 ? (I)gridDim.y * (kBinThreads / 32) : 1;
+  const I y_at = dims == 3 ? (I)lane : (I)blockIdx.y * kBinThreads + threadIdx.x;
+  const I y_by = dims == 3 ? 32 : (I)gridDim.y * kBinThreads;
+  const double sites = (double)N * (dims >= 2 ? (double)N : 1.0) * (dims == 3 ? (double)N : 1.0);
+  PowerSum sum;
+  unsigned long long count = 0;
+  for (I nz = zmin + z_at; nz <= zmax; nz += z_by)
+    for (I ny = ymin + y_at; ny <= ymax; ny += y_by) {
+      const I r2 = ny * ny + nz * nz;
+      if (r2 > last) continue;
+      const int hi = (int)min((I)isqrt(last - r2), half);
+      const I from = first - r2;
+      const int lo = from <= 0 ? 0 : isqrt(from - 1) + 1;         // ceil(sqrt(from))
+      const C* row = F + ((int64_t)(nz < 0 ? nz + N : nz) * N + (ny < 0 ? ny + N : ny)) * nx;
+      for (int ix = lo; ix <= hi; ++ix) {
+        const bool once = ix == 0 || (N % 2 == 0 && ix == half);
+        const C v = row[ix];
+        if (b == 0) sum.add((double)v.x + (double)f[0] * sites, (double)v.y, 1.0);   // S f(site 0)
+        else sum.add(v.x, v.y, (decltype(v.x))(once ? 1 : 2));
+        count += once ? 1 : 2;
+      }
     }
-    const int b = (int)floor(sqrt(n2) + 0.5);
-    if (b >= nbins) continue;
-    const double w = (ix == 0 || (N % 2 == 0 && ix == N / 2)) ? 1.0 : 2.0;
-    double re = (double)F[k].x;
-    const double im = (double)F[k].y;
-    if (k == 0) re += (double)f[0] * (double)(total / nx * N);  // S f(site 0)
-    atomicAdd(&hp[b], w * (re * re + im * im));
-    atomicAdd(&hn[b], w);
+  double p = sum.total();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    p += __shfl_down_sync(0xffffffffu, p, o);
+    count += __shfl_down_sync(0xffffffffu, count, o);
+  }
+  if (lane == 0) {
+    sp[warp] = p;
+    sn[warp] = count;
   }
   __syncthreads();
-  for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
-    part_p[(int64_t)blockIdx.x * nbins + b] = hp[b];
-    part_n[(int64_t)blockIdx.x * nbins + b] = hn[b];
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kBinThreads / 32; ++w) {
+      p += sp[w];
+      count += sn[w];
+    }
+    part_p[(int64_t)blockIdx.y * nbins + b] = p;
+    part_n[(int64_t)blockIdx.y * nbins + b] = (double)count;
   }
 }
 
-__global__ void k_spectrum_finalize(const double* __restrict__ part_p, const double* __restrict__ part_n, int blocks,
-                                    int nbins, double* __restrict__ p_out, double* __restrict__ n_out) {
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nbins; b += gridDim.x * blockDim.x) {
-    double p = 0.0, n = 0.0;
-    for (int k = 0; k < blocks; ++k) {  // fixed order over blocks
-      p += part_p[(int64_t)k * nbins + b];
-      n += part_n[(int64_t)k * nbins + b];
+// All bins at once, where a warp's histogram fits the shared memory: warps take rows
+// along x (read once, coalesced), along which the bin does not decrease, so a warp adds
+// the modes of a bin by shuffles between neighbouring lanes and the first lane of each
+// run adds the total to the warp's own histogram: nothing atomic, and a fixed order.
+// 256^3 FP32: 137 us, 212 for the kernel above, which reads single modes out of 32-byte
+// sectors; latency of the shuffles and of the histogram bounds it (HBM: 10 us), and
+// eight blocks an SM in place of four are no faster.  A whole spectrum at 256^3 FP32:
+// 761 -> 291 us, 64^3 173 -> 60, 4096^2 694 -> 317, 65536 161 -> 77.
+template <typename T>
+struct RowSum;
+template <>
+struct RowSum<float> {
+  static constexpr int bytes = 12;   // a pair and a count per bin and warp
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void take(const PowerSum& p) {
+    hi = p.hi;
+    lo = p.lo;
+  }
+  __device__ __forceinline__ void add_lane(int o, bool same) {
+    const float h = __shfl_down_sync(0xffffffffu, hi, o), l = __shfl_down_sync(0xffffffffu, lo, o);
+    if (same) {
+      lo += l;
+      ce::add_to(hi, lo, h);
     }
+  }
+  __device__ __forceinline__ void add_to_bin(float2* bin) const {
+    float2 x = *bin;
+    x.y += lo;
+    ce::add_to(x.x, x.y, hi);
+    *bin = x;
+  }
+  static __device__ __forceinline__ double value(const float2& x) { return (double)x.x + (double)x.y; }
+  using Bin = float2;
+};
+template <>
+struct RowSum<double> {
+  static constexpr int bytes = 12;
+  double v = 0.0;
+  __device__ __forceinline__ void take(const PowerSum& p) { v = p.wide; }
+  __device__ __forceinline__ void add_lane(int o, bool same) {
+    const double x = __shfl_down_sync(0xffffffffu, v, o);
+    if (same) v += x;
+  }
+  __device__ __forceinline__ void add_to_bin(double* bin) const { *bin += v; }
+  static __device__ __forceinline__ double value(double x) { return x; }
+  using Bin = double;
+};
+
+constexpr int kBinWarps = kBinThreads / 32;
+inline size_t rows_smem(int nbins) { return (size_t)nbins * (8 + kBinWarps * 12); }
+
+template <typename C, typename T>
+__global__ void __launch_bounds__(kBinThreads) k_bin_rows(const C* __restrict__ F, const T* __restrict__ f, int N,
+                                                           int dims, int nbins, double* __restrict__ part_p,
+                                                           double* __restrict__ part_n) {
+  using Bin = typename RowSum<T>::Bin;
+  extern __shared__ __align__(16) unsigned char hist[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double* wide = reinterpret_cast<double*>(hist);            // values outside the pairs' range, the whole block's
+  Bin* bins = reinterpret_cast<Bin*>(wide + nbins);          // [warp][bin]
+  unsigned* counts = reinterpret_cast<unsigned*>(bins + (size_t)kBinWarps * nbins);
+  for (int b = threadIdx.x; b < nbins; b += kBinThreads) wide[b] = 0.0;
+  for (int b = threadIdx.x; b < kBinWarps * nbins; b += kBinThreads) {
+    bins[b] = Bin{};
+    counts[b] = 0u;
+  }
+  __syncthreads();
+  Bin* mine = bins + (size_t)warp * nbins;
+  unsigned* mine_n = counts + (size_t)warp * nbins;
+  const int half = N / 2, nx = half + 1, rows = dims == 3 ? N * N : N;
+  const double sites = (double)N * (double)N * (dims == 3 ? (double)N : 1.0);
+  for (int row = blockIdx.x * kBinWarps + warp; row < rows; row += gridDim.x * kBinWarps) {
+    int ny = row % N, nz = row / N;
+    ny = ny <= half ? ny : ny - N;
+    nz = nz <= half ? nz : nz - N;
+    const int r2 = ny * ny + nz * nz;
+    const C* at = F + (int64_t)row * nx;
+    for (int x0 = 0; x0 <= half; x0 += 32) {
+      const int ix = x0 + lane, n2 = r2 + ix * ix, root = isqrt(n2);
+      const int b = ix <= half ? root + (n2 > root * root + root) : 0x7fffffff;
+      const bool in = b < nbins;
+      const int w = ix == 0 || (N % 2 == 0 && ix == half) ? 1 : 2;
+      PowerSum p;
+      if (in) {
+        const C v = at[ix];
+        if (n2 == 0) p.add((double)v.x + (double)f[0] * sites, (double)v.y, 1.0);   // S f(site 0)
+        else p.add(v.x, v.y, (decltype(v.x))w);
+        if (sizeof(T) == 4 && p.wide != 0.0) atomicAdd(wide + b, p.wide);   // also NaN
+      }
+      RowSum<T> s;
+      s.take(p);
+      int n = in ? w : 0;
+      for (int o = 1; o < 32; o *= 2) {
+        const int other = __shfl_down_sync(0xffffffffu, b, o);
+        const bool same = lane + o < 32 && other == b;
+        if (!__any_sync(0xffffffffu, same)) break;
+        s.add_lane(o, same);
+        const int m = __shfl_down_sync(0xffffffffu, n, o);
+        n += same ? m : 0;
+      }
+      const int before = __shfl_up_sync(0xffffffffu, b, 1);
+      if (in && (lane == 0 || before != b)) {
+        s.add_to_bin(mine + b);
+        mine_n[b] += (unsigned)n;
+      }
+      __syncwarp();   // the next 32 modes may begin in this bin
+      if (__shfl_sync(0xffffffffu, b, 31) >= nbins) break;   // no later mode of the row is in a bin
+    }
+  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < nbins; b += kBinThreads) {
+    double p = wide[b], n = 0.0;
+    for (int w = 0; w < kBinWarps; ++w) {
+      p += RowSum<T>::value(bins[(size_t)w * nbins + b]);
+      n += (double)counts[(size_t)w * nbins + b];
+    }
+    part_p[(int64_t)blockIdx.x * nbins + b] = p;
+    part_n[(int64_t)blockIdx.x * nbins + b] = n;
+  }
+}
+
+// Bins the half spectrum F into `parts` partial histograms of nbins (at most kBinParts).
+template <typename C, typename T>
+cudaError_t bin_spectrum(cudaStream_t st, int sms, const void* F, const void* f, int64_t N, int dims, int nbins,
+                         double* part_p, double* part_n, int* parts) {
+  const C* Fc = static_cast<const C*>(F);
+  const T* ft = static_cast<const T*>(f);
+  // n^2 <= dims (N/2)^2, and b^2 + b a little above: exact in a float?
+  const bool small = (double)dims * (double)(N / 2 + 2) * (double)(N / 2 + 2) < 16e6;
+  const size_t shm = rows_smem(nbins);
+  if (dims >= 2 && small && shm <= kRowsSmem) {
+    const int rows = (int)(dims == 3 ? N * N : N);
+    const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(4, kRowsSmem / shm));
+    *parts = std::min(std::min(kBinParts, per_sm * sms), (rows + kBinWarps - 1) / kBinWarps);
+    const cudaError_t e = cudaFuncSetAttribute(k_bin_rows<C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem);
+    if (e != cudaSuccess) return e;
+    k_bin_rows<C, T><<<*parts, kBinThreads, shm, st>>>(Fc, ft, (int)N, dims, nbins, part_p, part_n);
+    return cudaGetLastError();
+  }
+  // rows of a bin per block: eight planes' worth of nz (3D), 1024 rows (2D)
+  *parts = dims == 1 ? 1 : (int)std::min<int64_t>(kBinChunks, dims == 3 ? (N + 31) / 32 : (N + 1023) / 1024);
+  const dim3 grid(nbins, *parts);
+  if (small) k_bin_spectrum<C, T, int><<<grid, kBinThreads, 0, st>>>(Fc, ft, N, dims, nbins, part_p, part_n);
+  else k_bin_spectrum<C, T, int64_t><<<grid, kBinThreads, 0, st>>>(Fc, ft, N, dims, nbins, part_p, part_n);
+  return cudaGetLastError();
+}
+
+// One warp per bin: lanes take parts l, l + 32, ..., then a fixed shuffle tree.
+__global__ void k_spectrum_finalize(const double* __restrict__ part_p, const double* __restrict__ part_n, int parts,
+                                    int nbins, double* __restrict__ p_out, double* __restrict__ n_out) {
+  const int lane = threadIdx.x & 31, b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (b >= nbins) return;
+  double p = 0.0, n = 0.0;
+  for (int k = lane; k < parts; k += 32) {
+    p += part_p[(int64_t)k * nbins + b];
+    n += part_n[(int64_t)k * nbins + b];
+  }
+  p = ce::warp_sum(p);
+  n = ce::warp_sum(n);
+  if (lane == 0) {
     p_out[b] = n > 0.0 ? p / n : 0.0;
     n_out[b] = n;
   }
@@ -146,6 +363,9 @@ SpectrumWork* find_work(const ce_sim* s, bool create) {
   work_table().push_back({s, SpectrumWork{}});
   return &work_table().back().second;
 }
+
+// Partial histograms a handle's work buffers hold.
+int spectrum_parts(const ce_sim* s) { return s->dims == 1 ? kBinChunks : kBinParts; }
 
 constexpr char kMagic[8] = {'C', 'E', 'G', 'R', 'I', 'D', '0', '1'};
 
@@ -201,7 +421,7 @@ int ce_spectrum(ce_sim* s, int field, int nbins, double* k, double* power, doubl
     w->have_plan = true;
     e = cudaMalloc(&w->spec, (size_t)half * (f32 ? sizeof(cufftComplex) : sizeof(cufftDoubleComplex)));
     if (e == cudaSuccess) e = cudaMalloc(&w->real, (size_t)s->S * s->esize);
-    if (e == cudaSuccess) e = cudaMalloc(&w->part, sizeof(double) * 2 * kBinBlocks * max_bins);
+    if (e == cudaSuccess) e = cudaMalloc(&w->part, sizeof(double) * 2 * spectrum_parts(s) * max_bins);
     if (e == cudaSuccess) e = cudaMalloc(&w->out, sizeof(double) * 2 * max_bins);
     if (e != cudaSuccess) {
       ce::outputs_release(s);
@@ -226,20 +446,15 @@ int ce_spectrum(ce_sim* s, int field, int nbins, double* k, double* power, doubl
     r = cufftExecD2Z(w->plan, static_cast<cufftDoubleReal*>(w->real), static_cast<cufftDoubleComplex*>(w->spec));
   if (r != CUFFT_SUCCESS) return ofail(CE_ECUDA, "ce_spectrum: cufft exec failed");
   double* part_p = w->part;
-  double* part_n = w->part + (int64_t)kBinBlocks * nbins;
-  const size_t shm = sizeof(double) * 2 * nbins;
-  if (f32)
-    k_bin_spectrum<cufftComplex, float><<<kBinBlocks, kBinThreads, shm, s->stream>>>(
-        static_cast<const cufftComplex*>(w->spec), static_cast<const float*>(s->f[s->cur][field]), s->N, s->dims,
-        nbins, part_p, part_n);
-  else
-    k_bin_spectrum<cufftDoubleComplex, double><<<kBinBlocks, kBinThreads, shm, s->stream>>>(
-        static_cast<const cufftDoubleComplex*>(w->spec), static_cast<const double*>(s->f[s->cur][field]), s->N,
-        s->dims, nbins, part_p, part_n);
-  e = cudaGetLastError();
+  double* part_n = w->part + (int64_t)spectrum_parts(s) * nbins;
+  int parts = 1;
+  const void* field_data = s->f[s->cur][field];
+  e = f32 ? bin_spectrum<cufftComplex, float>(s->stream, s->sms, w->spec, field_data, s->N, s->dims, nbins, part_p,
+                                              part_n, &parts)
+          : bin_spectrum<cufftDoubleComplex, double>(s->stream, s->sms, w->spec, field_data, s->N, s->dims, nbins,
+                                                     part_p, part_n, &parts);
   if (e != cudaSuccess) return ocuda(e, "ce_spectrum: binning");
-  k_spectrum_finalize<<<(nbins + 127) / 128, 128, 0, s->stream>>>(part_p, part_n, kBinBlocks, nbins, w->out,
-                                                                   w->out + nbins);
+  k_spectrum_finalize<<<(nbins + 7) / 8, 256, 0, s->stream>>>(part_p, part_n, parts, nbins, w->out, w->out + nbins);
   std::vector<double> host(2 * (size_t)nbins);
   e = cudaMemcpyAsync(host.data(), w->out, sizeof(double) * 2 * nbins, cudaMemcpyDeviceToHost, s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
