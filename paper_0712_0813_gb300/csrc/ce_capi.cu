@@ -525,18 +525,21 @@ int ce_create(const ce_config* cfg, ce_sim** out) {
       s->kernel = CE_KERNEL_GENERIC;   // automatic choice: fall back to the generic kernel
     }
   }
-  if (cfg->kernel == CE_KERNEL_AUTO && !sweep_hinted && !(cfg->flags & CE_FLAG_TEST_TMA_STALL)) {
+  // Not an expanding FP32 run of one field: the resident kernel groups the energy sums
+  // otherwise, so float(c) and then every site's rounding part after some hundred steps.
+  // Both are as near to the exact state, but with a single field the variance and G are
+  // read from fluctuations of 1e-2 about 1 and show the difference (up to 3e-4 after
+  // 1000 steps; with more fields below 1e-6).
+  const bool rounding_shows = s->prec == CE_F32 && s->nf == 1 && s->cfg.expansion;
+  if (cfg->kernel == CE_KERNEL_AUTO && !sweep_hinted && !rounding_shows && !(cfg->flags & CE_FLAG_TEST_TMA_STALL)) {
     s->res = s->prec == CE_F32 ? ce::resident_plan_f32(s->dims, s->N, s->nf, s->device, s->sms)
                                : ce::resident_plan_f64(s->dims, s->N, s->nf, s->device, s->sms);
     if (s->res.blocks > 0) {
       const size_t bytes = kResidentCounterWords * sizeof(unsigned) + (size_t)s->res.blocks * 2 * sizeof(double);
       s->res_counter = static_cast<unsigned*>(dalloc(s, bytes));
       if (!s->res_counter) {
-        ce_free(s);
-        return fail(CE_ENOMEM, "ce_create: device allocation of scratch failed");
-      }
-      e = cudaMemsetAsync(s->res_counter, 0, bytes, s->stream);
-      if (e != cudaSuccess) {
+        s->res = ce::ResidentPlan{};   // no room for it: one launch a step
+      } else if ((e = cudaMemsetAsync(s->res_counter, 0, bytes, s->stream)) != cudaSuccess) {
         ce_free(s);
         return cuda_fail(e, "ce_create: init");
       }

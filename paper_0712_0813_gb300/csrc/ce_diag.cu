@@ -215,6 +215,37 @@ __device__ __forceinline__ void diag_outputs(const DiagArgs<T>& p, int blocks) {
   if (!isfinite(E)) atomicCAS(&p.aux->status, CE_OK, CE_ENONFINITE);
 }
 
+// End of a launch: the block's sums (the first NS quantities; zero beyond), and in the
+// last block the outputs.
+template <typename T, int NF, int NS>
+__device__ __forceinline__ void diag_finish(const DiagArgs<T>& p, RunningSums<T, NS>& acc, double* big) {
+  constexpr int NV = 4 * NF + 1;
+  __shared__ double red[kDiagWarps][NS];
+  __shared__ int s_last;
+#pragma unroll
+  for (int j = 0; j < NS; ++j) {
+    const double v = acc.warp_total(j);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][j] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < NV) {
+    double t = 0.0;
+    if (threadIdx.x < NS) {
+      t = big[threadIdx.x];
+      for (int w = 0; w < kDiagWarps; ++w) t += red[w][threadIdx.x];
+    }
+    p.partials[(int64_t)blockIdx.x * NV + threadIdx.x] = t;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&p.aux->counter_diag, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  diag_outputs<T, NF>(p, gridDim.x);
+  if (threadIdx.x == 0) p.aux->counter_diag = 0u;
+}
+
 template <typename T, int NF, int DIMS>
 __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 1) k_diag(const DiagArgs<T> p, const DiagTasks tk) {
   constexpr int NV = 4 * NF + 1;
@@ -222,8 +253,7 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 
   const int64_t N = p.N;
   const DiagScalars<T> k = diag_scalars(p);
   const int raw_u = p.raw_u;
-  __shared__ double red[kDiagWarps][NV], big[NV];
-  __shared__ int s_last;
+  __shared__ double big[NV];
   if (threadIdx.x < NV) big[threadIdx.x] = 0.0;
   __syncthreads();
   RunningSums<T, NV> acc;
@@ -321,25 +351,89 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 
       acc.add(part, big);
     }
   }
+  diag_finish<T, NF, NV>(p, acc, big);
+}
+
+// Energies of an expanding FP32 run's starting state (w is u), from which a'(0) and
+// a''(0) follow and with them float(c) of every step.  What a thread adds in FP32 is 16
+// sites at the grid's stride: any other 16 are as near to the exact sums (1e-8), but
+// float(c) would round otherwise now and then, and from then on every site's rounding,
+// so a run would end off by its own rounding error (2e-5 of the velocities after 1000
+// steps).  No field moments.
+template <int NF, int DIMS>
+__global__ void __launch_bounds__(kDiagThreads, NF <= 2 ? 4 : 2) k_start_sums(const DiagArgs<float> p) {
+  constexpr int NV = 2 * NF + 1;
+  __shared__ double big[NV];
+  if (threadIdx.x < NV) big[threadIdx.x] = 0.0;
+  __syncthreads();
+  RunningSums<float, NV> acc;
+  acc.clear();
+  const int64_t N = p.N, stride = (int64_t)gridDim.x * kDiagThreads;
+  const int64_t plane = DIMS == 3 ? N * N : N;
+  int64_t s = (int64_t)blockIdx.x * kDiagThreads + threadIdx.x;
+  // coordinates of s and of the stride (1D: x is s)
+  const int n = DIMS == 1 ? 0 : (int)N;
+  int x = 0, y = 0, z = 0, dx = 0, dy = 0, dz = 0;
+  if constexpr (DIMS >= 2) {
+    x = (int)(s % N);
+    dx = (int)(stride % N);
+    y = (int)(DIMS == 3 ? s / N % N : s / N);
+    dy = (int)(DIMS == 3 ? stride / N % N : stride / N);
+  }
+  if constexpr (DIMS == 3) {
+    z = (int)(s / plane);
+    dz = (int)(stride / plane);
+  }
+  const float q[3] = {(float)p.q[0], (float)p.q[1], (float)p.q[2]};
+  const int64_t groups = ((p.S + stride - 1) / stride + kFlush - 1) / kFlush;
+  for (int64_t g = 0; g < groups; ++g) {
+    float part[NV];
 #pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    const double v = acc.warp_total(j);
-    if (lane == 0) red[warp][j] = v;
+    for (int j = 0; j < NV; ++j) part[j] = 0.f;
+#pragma unroll 4
+    for (int r = 0; r < kFlush; ++r) {
+      if (s >= p.S) break;
+      int64_t up[DIMS];   // the neighbours at +e_d
+      up[0] = (DIMS == 1 ? s == N - 1 : x == n - 1) ? s - (N - 1) : s + 1;
+      if constexpr (DIMS >= 2) up[1] = y == n - 1 ? s - (N - 1) * N : s + N;
+      if constexpr (DIMS == 3) up[2] = z == n - 1 ? s - (N - 1) * plane : s + plane;
+      float f[NF], dv[NF], vs;
+#pragma unroll
+      for (int i = 0; i < NF; ++i) {
+        f[i] = __ldg(p.f[i] + s);
+        const float u = __ldg(p.w[i] + s);
+        float g2 = 0.f;
+#pragma unroll
+        for (int d = 0; d < DIMS; ++d) {
+          const float df = __ldg(p.f[i] + up[d]) - f[i];
+          g2 = fmaf(df, df, g2);
+        }
+        part[i] = fmaf(0.5f * u, u, part[i]);
+        part[NF + i] += g2;
+      }
+      model_dv<float, NF>(f, q, dv, vs);
+      part[2 * NF] += vs;
+      s += stride;
+      if constexpr (DIMS >= 2) {   // in range again after one subtraction each
+        x += dx;
+        y += dy;
+        if (x >= n) {
+          x -= n;
+          ++y;
+        }
+      }
+      if constexpr (DIMS == 3) {
+        z += dz;
+        if (y >= n) {
+          y -= n;
+          ++z;
+        }
+      }
+    }
+    __syncwarp();
+    acc.add(part, big);
   }
-  __syncthreads();
-  if (threadIdx.x < NV) {
-    double t = big[threadIdx.x];
-    for (int w = 0; w < kDiagWarps; ++w) t += red[w][threadIdx.x];
-    p.partials[(int64_t)blockIdx.x * NV + threadIdx.x] = t;
-    __threadfence();
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&p.aux->counter_diag, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  diag_outputs<T, NF>(p, gridDim.x);
-  if (threadIdx.x == 0) p.aux->counter_diag = 0u;
+  diag_finish<float, NF, NV>(p, acc, big);
 }
 
 // A grid that is resident as a whole (at most `cap` blocks): tasks are strided.
@@ -350,6 +444,13 @@ cudaError_t launch_diag_dims(const DiagArgs<T>& a, int cap, cudaStream_t st) {
       per_sm < 1) {
     cudaGetLastError();
     per_sm = 1;
+  }
+  if constexpr (sizeof(T) == 4) {
+    if (a.raw_u && a.expansion) {
+      const int blocks = (int)std::min<int64_t>((a.S + kDiagThreads - 1) / kDiagThreads, cap);
+      k_start_sums<NF, DIMS><<<blocks, kDiagThreads, 0, st>>>(a);
+      return cudaGetLastError();
+    }
   }
   cap = std::min(cap, per_sm * sm_count(-1));
   const DiagTasks tk = diag_tasks(DIMS, a.N, a.S, cap);
