@@ -49,6 +49,21 @@ __device__ __forceinline__ void stcs16v(T* p, const T (&o)[VX]) {
   }
 }
 
+// A value at a 32-bit byte offset from a base that is the same for the whole warp: the
+// base stays in uniform registers and the access needs no 64-bit address arithmetic.
+template <typename T>
+__device__ __forceinline__ T ldg_at(const T* base, uint32_t bytes) {
+  return __ldg(reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + bytes));
+}
+template <typename T>
+__device__ __forceinline__ void st_at(T* base, uint32_t bytes, T v) {
+  *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + bytes) = v;
+}
+template <typename T>
+__device__ __forceinline__ void stcs_at(T* base, uint32_t bytes, T v) {
+  __stcs(reinterpret_cast<T*>(reinterpret_cast<char*>(base) + bytes), v);
+}
+
 // One 16-byte group of the 1D step: VX = 16 / sizeof(T) consecutive sites
 // starting at site s = k VX of a periodic 1D lattice of N sites (N a multiple
 // of VX), all fields.  16-byte loads of the group's f and w, scalar loads of the

@@ -33,7 +33,7 @@ constexpr int kLineThreads = 32 * kLineWarps;
 constexpr int kStrip = 30;   // sites a warp updates along x
 
 // rows of loads in flight per lane (6001^2, 2 fields: 4 rows 229.0 us, 6 rows
-// 223.8, 8 rows 228.9, the last at 3 instead of 4 blocks per SM; 16001^2: 1642,
+// 223.8 (219 now), 8 rows 228.9, the last at 3 instead of 4 blocks per SM; 16001^2: 1642,
 // 1497, 1541 us)
 template <int NF>
 struct LineDepth {
@@ -57,11 +57,14 @@ __global__ void __launch_bounds__(kLineThreads) k_step_lines(const StepArgs<T> p
     const int n = y1 - y0 + 2;                                 // rows y0 - 1 .. y1
     const bool down = (blockIdx.y & 1u) != 0;
     // row k of the sweep: y0 - 1 + k upwards, y1 - k downwards (mod N)
-    const auto row_off = [&](int k) -> int64_t {
+    const auto row_off = [&](int k) -> int64_t {   // the same for the whole block (NF > 1)
       int64_t y = down ? (int64_t)y1 - k : (int64_t)y0 - 1 + k;
       y = y < 0 ? y + N : (y >= N ? y - N : y);
-      return y * N + xs;
+      return y * N + (NF == 1 ? xs : 0);
     };
+    // the lane's column in bytes; one field has few enough addresses to keep whole
+    // (6001^2: 161 us, 178 with the offset; two fields, without and with it, 227 and 219)
+    const uint32_t xb = NF == 1 ? 0u : (uint32_t)xs * (uint32_t)sizeof(T);
     const T c = (T)p.sc_in->c;
     const T dd = p.dt_drift, kk = p.dt_kick, idx2 = p.inv_dx2;
     const T q[3] = {p.q[0], p.q[1], p.q[2]};
@@ -70,8 +73,8 @@ __global__ void __launch_bounds__(kLineThreads) k_step_lines(const StepArgs<T> p
       const int64_t o = row_off(k);
 #pragma unroll
       for (int i = 0; i < NF; ++i) {
-        lf[slot][i] = __ldg(p.f_in[i] + o);
-        lw[slot][i] = __ldg(p.w_in[i] + o);
+        lf[slot][i] = ldg_at(p.f_in[i] + o, xb);
+        lw[slot][i] = ldg_at(p.w_in[i] + o, xb);
       }
     };
 #pragma unroll
@@ -125,8 +128,8 @@ __global__ void __launch_bounds__(kLineThreads) k_step_lines(const StepArgs<T> p
           const int64_t o = row_off(j - 1);
 #pragma unroll
           for (int i = 0; i < NF; ++i) {
-            __stcs(p.w_out[i] + o, fmaT(kk, lap[i] - dv[i], vc[i]));
-            __stcs(p.f_out[i] + o, gc[i]);
+            stcs_at(p.w_out[i] + o, xb, fmaT(kk, lap[i] - dv[i], vc[i]));
+            stcs_at(p.f_out[i] + o, xb, gc[i]);
           }
         }
         if (++since_flush == 16) {
