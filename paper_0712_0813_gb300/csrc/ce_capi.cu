@@ -650,6 +650,11 @@ int ce_step(ce_sim* s, int64_t n) {
     while (n > 0 && cap == cudaStreamCaptureStatusNone) {
       const int m = (int)std::min<int64_t>(n, kResidentSteps);
       e = s->prec == CE_F32 ? launch_resident_steps<float>(s, s->cur, m) : launch_resident_steps<double>(s, s->cur, m);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {   // a stream that may use part of the GPU only
+        cudaGetLastError();
+        s->res = ce::ResidentPlan{};                   // one launch a step from here on
+        break;
+      }
       if (e != cudaSuccess) return cuda_fail(e, "ce_step: launch");
       s->res_count += (uint32_t)m * (uint32_t)s->res.blocks;
       s->cur ^= m & 1;
