@@ -302,24 +302,26 @@ def roofline_of(w, precision, ms_per_step, hbm_peak, peak_kind, kernel):
     return out
 
 
-# FP64 instructions per site of the generic kernel's two-pass FP64 step, 3D, 2
-# fields (ncu, 256^3: k_drift_g 2 per field and site, k_kick_from_g 14.1; each
-# DADD, DMUL or DFMA takes one slot of the FP64 pipe), and the pipe's rate:
+# FP64 instructions per site of a 3D, 2-field FP64 step (each DADD, DMUL or DFMA
+# takes one slot of the FP64 pipe): with all of its arithmetic in FP64, each site's
+# g formed once, and of the automatic kernel, which forms the force in integers
+# (both counted by ncu at 256^3, halo lanes included).  The pipe's rate:
 # GB300's nominal FP64 1.25 TFLOP/s counts a DFMA as 2 flops, so 0.625 T
 # instructions/s (152 SMs x 2 FP64 lanes x 2.07 GHz = 0.629 T).
 FP64_OPS_PER_SITE_2F_3D = 32.2
+FP64_OPS_PER_SITE_2F_3D_INTEGER_FORCE = 10.2
 FP64_PIPE_PEAK_TOPS = 0.625
 
 
-def fp64_alu_roofline(w, gsites_per_s: float, kernel: str, hbm_peak: float):
-    """The plain FP64 path is bound by GB300's FP64 pipe, not by HBM: its
-    roofline in FP64 instructions per second (2-field 3D lattices on the generic
-    kernel's two passes, whose per-site count was measured)."""
+def fp64_alu_roofline(w, gsites_per_s: float, kernel: str, hbm_peak: float,
+                      ops_per_site: float = FP64_OPS_PER_SITE_2F_3D):
+    """FP64 steps against GB300's FP64 pipe: FP64 instructions per second (2-field
+    3D lattices on CE_KERNEL_GENERIC, whose per-site counts are known)."""
     if not (w["dims"] == 3 and w["nf"] == 2 and kernel == "generic"):
         return None
-    achieved = gsites_per_s * FP64_OPS_PER_SITE_2F_3D / 1e3
+    achieved = gsites_per_s * ops_per_site / 1e3
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PIPE_PEAK_TOPS, "unit": "T FP64 instructions/s",
-            "frac": achieved / FP64_PIPE_PEAK_TOPS, "ops_per_site": FP64_OPS_PER_SITE_2F_3D,
+            "frac": achieved / FP64_PIPE_PEAK_TOPS, "ops_per_site": ops_per_site,
             "peak_kind": "nominal FP64 rate (1.25 TFLOP/s, a DFMA = 2 flops = one pipe slot)",
             "hbm_frac": gsites_per_s * 4 * 8 * w["nf"] / hbm_peak}
 
@@ -756,7 +758,7 @@ def main():
         r_, s_, z_ = (int(x) for x in args.plan.split(","))
         hints = {"tile_rows": r_, "stages": s_, "zchunks": z_}
     elif not args.no_autotune and w["dims"] == 3 and args.precision == "f32":
-        tune = True   # (FP64 keeps the automatic choice: the generic kernel's two passes, faster in FP64)
+        tune = True   # (FP64 keeps the automatic choice: the one-pass kernel with the force in integers, faster in FP64)
     ms, kernel, clocks, plan, tune_info = time_device_steps(
         capi, torch, w, f0, u0, args.precision, args.steps, args.warmup, barrier,
         sampler_gpu=gpu_index if rank == 0 else None, hints=hints, tune=tune)
@@ -768,8 +770,9 @@ def main():
     secs = ms / 1e3
     value = replicas.aggregate_throughput(ws, S * args.steps, secs) / 1e9
     roofline = roofline_of(w, args.precision, ms / args.steps, hbm_peak, peak_kind, kernel)
-    if args.precision == "f64":   # bound by the FP64 pipe, not by HBM: that roofline when it is known
-        roofline = fp64_alu_roofline(w, value / ws, kernel, hbm_peak) or roofline   # per GPU
+    if args.precision == "f64":   # not HBM's: the FP64 pipe's roofline where the count is known
+        roofline = fp64_alu_roofline(w, value / ws, kernel, hbm_peak,   # per GPU
+                                     FP64_OPS_PER_SITE_2F_3D_INTEGER_FORCE) or roofline
 
     # plain FP64 path on the same lattice: the library's automatic FP64 choice
     w64 = min(args.warmup, 5)
@@ -840,7 +843,8 @@ def main():
                        "l2": f"state {4 * esize * w['nf'] * S / 1e6:.0f} MB > L2 (129 MB); no flush needed"},
             "fp64_plain": {"value": value64, "ms_per_step": ms64 / args.fp64_steps, "steps": args.fp64_steps,
                            "kernel": kernel64, "sweep_plan": list(plan64), "f32_over_f64": value / value64,
-                           "roofline": fp64_alu_roofline(w, value64 / ws, kernel64, hbm_peak)},
+                           "roofline": fp64_alu_roofline(w, value64 / ws, kernel64, hbm_peak,
+                                                         FP64_OPS_PER_SITE_2F_3D_INTEGER_FORCE)},
             "roofline": roofline,
             "fp32_vs_fp64": fp32_vs_fp64,
             "cube256": cube256,
