@@ -8,8 +8,11 @@
 //   sum of the energy terms (expansion only)         1 FP64 operation a site
 // What bounds it.  GB300 has two FP64 lanes per clock and SM, so the step in FP64
 // (a pass for g, a pass for the stencil, 32 operations a site with two fields) ran
-// at 0.85 of that pipe and 0.15 of HBM.  Here 9.4 FP64 operations a site remain
-// (halo rows included) beside ~350 integer instructions on the other pipes.
+// at 0.85 of that pipe and 0.15 of HBM.  Here 10.2 FP64 operations a site remain
+// (256^3 by ncu, halo lanes included; half of that pipe) among 782 instructions, most
+// of them integer.  596 us a step at 256^3 (two passes: 1058), 30.9 ms at 1024^3 (67):
+// bound by issue and its latency, 0.60 of the issue slots with 17 warps an SM (96
+// registers a thread), beside 0.27 of HBM.
 //
 // Layout.  3D: the column kernel's (ce_cols3d.cu): a warp owns 30 x-sites by TY
 // rows and sweeps a chunk of z; lane l holds column x0 - 1 + l, so lanes 0 and
