@@ -11,8 +11,9 @@
 // site's neighbours are aligned to the largest exponent among them, so what
 // alignment drops of each is below 2^-57 of the largest value of the stencil, where
 // FP64 rounds every partial sum to 2^-53 of it; products are the upper 64 bits of
-// unsigned 64-bit fractions (7 instructions; a signed one takes 17).  The force is thus at least as accurate as FP64's, site by site, whatever the
-// field's range.  Non-finite values are left to the caller (fx_finite).
+// unsigned 64-bit fractions (7 instructions; a signed one takes 17), and the two meet
+// in a unit 2^-54 of the model force or 2^-61 of the Laplacian.  The force is thus at
+// least as accurate as FP64's, site by site, whatever the field's range.  Non-finite values are left to the caller (fx_finite).
 //
 // Plain C++ apart from the shift and the bit casts, so the CPU tests compile it.
 #pragma once
@@ -79,7 +80,18 @@ CE_FX_HD int64_t asr(int64_t x, int s) {
 #endif
 }
 
-// The same, to nearest.
+// x << s, s >= 0 of any size.
+CE_FX_HD int64_t shl(int64_t x, int s) {
+#ifdef __CUDA_ARCH__
+  int64_t r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(s));
+  return r;
+#else
+  return s > 63 ? 0 : (int64_t)((uint64_t)x << s);
+#endif
+}
+
+// x >> s, to nearest.
 CE_FX_HD int64_t asr_round(int64_t x, int s) {
   const int64_t r = asr(x, s - 1 < 0 ? 0 : s - 1);
   return s > 0 ? (r + 1) >> 1 : r;
@@ -94,6 +106,7 @@ CE_FX_HD int clz64(uint64_t x) {
 }
 
 CE_FX_HD int imax(int a, int b) { return a > b ? a : b; }
+CE_FX_HD int imin(int a, int b) { return a < b ? a : b; }
 
 CE_FX_HD Fx from_double(double x) {
   const int64_t b = bits_of(x);
@@ -244,6 +257,10 @@ CE_FX_HD int64_t lsr_round(uint64_t x, int s) { return (int64_t)((lsr(x, s - 1) 
 // energy terms with their signs turned: callers alternate it from lane to lane,
 // so that what rounding downwards adds to the terms (1e-15 of the sum, as a bias)
 // cancels over the lattice.
+// raw is moved up to the 62 bits it may fill, as far as the model force's own unit
+// allows, before the two meet: on a fine or smooth lattice raw is far below its
+// operands, and in their unit (2^-57 of g) the model force of a homogeneous field was
+// off by 2^-58 / dx^2, the same way at every site (1e-10 of it at dx^2 = 1e-7).
 template <int NF, int DIMS, bool SUMS, bool FAST>
 CE_FX_HD void site_force(const Fx (&g)[NF], const Fx (&nb)[NF][2 * DIMS], const int (&em)[NF],
                          const SiteModel<NF>& s, int flip, double (&force)[NF], double& energy) {
@@ -258,16 +275,23 @@ CE_FX_HD void site_force(const Fx (&g)[NF], const Fx (&nb)[NF][2 * DIMS], const 
 #pragma unroll
     for (int j = 0; j < 2 * DIMS; ++j) raw += asr(nb[i][j].m, em[i] - nb[i][j].e);
     const int ur = em[i] - kOne;
+    // |raw| <= 3 2^60: at least two leading bits free (zero: as far as the model force likes)
+    const int up = imin(raw == 0 ? 8192 : clz64((uint64_t)(raw ^ (raw >> 63))) - 2, ur - s.ud[i] - 2);
+    int u;
     if constexpr (FAST) {
-      force[i] = scaled<false>(raw - negate_if(lsr_round(s.d[i], ur - s.ud[i]), sign), ur);
+      raw = shl(raw, up);
+      u = ur - up;
+      force[i] = scaled<false>(raw - negate_if(lsr_round(s.d[i], u - s.ud[i]), sign), u);
     } else {   // the model force may be the coarser one
-      const int u = imax(ur, s.ud[i] + 2);
-      force[i] = scaled<true>(asr_round(raw, u - ur) - negate_if(lsr_round(s.d[i], u - s.ud[i]), sign), u);
+      const int v = ur - up;   // the common unit
+      raw = shl(raw, imax(up, 0));
+      u = ur - imax(up, 0);
+      force[i] = scaled<true>(asr_round(raw, v - u) - negate_if(lsr_round(s.d[i], v - s.ud[i]), sign), v);
     }
     if constexpr (SUMS) {
       const int64_t m = sign ^ flip;
       z[i] = mul_signed(s.x[i], negate_if(raw, m));        // (-)|g| sign(g) raw
-      uz[i] = s.ex[i] + ur;
+      uz[i] = s.ex[i] + u;
     }
   }
   if constexpr (SUMS) {
