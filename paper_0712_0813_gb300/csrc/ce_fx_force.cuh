@@ -20,12 +20,18 @@ static __device__ __noinline__ void force_fp64(const double* g, const double* nb
     double raw = -2.0 * DIMS * gs[i];
     for (int j = 0; j < 2 * DIMS; ++j) raw += nb[i * 2 * DIMS + j];
     force[i] = fma(-dx2, dv[i], raw);
-    e += gs[i] * fma(-0.75 * dx2, dv[i], raw);
+    if constexpr (DIMS == 1) {
+      const double df = nb[i * 2 + 1] - gs[i];
+      e -= df * df;
+    } else {
+      e += gs[i] * fma(-0.75 * dx2, dv[i], raw);
+    }
   }
-  *energy = e;
+  *energy = DIMS == 1 ? fma(-3.0 * dx2, vs, e) : e;
 }
 
-// The site's force by the form its values allow.
+// The site's force by the form its values allow.  In 1D the energy term is that of
+// line_energy, with its sign turned.
 template <int NF, int DIMS, bool SUMS>
 __device__ __forceinline__ void force_of(const Fx (&g)[NF], const Fx (&nb)[NF][2 * DIMS], const FxModel& k,
                                          double inv_dx2, const double (&q)[3], double (&force)[NF], double& energy) {
@@ -34,15 +40,21 @@ __device__ __forceinline__ void force_of(const Fx (&g)[NF], const Fx (&nb)[NF][2
   stencil_exponents<NF, DIMS>(g, nb, em);
   SiteModel<NF> s;
   site_model<NF, SUMS>(g, k, s);
+  Fx up[NF];
+#pragma unroll
+  for (int i = 0; i < NF; ++i) up[i] = nb[i][1];
+  constexpr bool kParts = SUMS && DIMS > 1;
   if (fast_site<NF>(em, s)) {
-    site_force<NF, DIMS, SUMS, true>(g, nb, em, s, flip, force, energy);
+    site_force<NF, DIMS, kParts, true>(g, nb, em, s, flip, force, energy);
+    if constexpr (SUMS && DIMS == 1) energy = -line_energy<NF>(g, up, s);
     return;
   }
   int most = em[0];
 #pragma unroll
   for (int i = 1; i < NF; ++i) most = max(most, em[i]);
   if (most < kNonFinite) {
-    site_force<NF, DIMS, SUMS, false>(g, nb, em, s, flip, force, energy);
+    site_force<NF, DIMS, kParts, false>(g, nb, em, s, flip, force, energy);
+    if constexpr (SUMS && DIMS == 1) energy = -line_energy<NF>(g, up, s);
     return;
   }
   double gd[NF], nd[NF * 2 * DIMS], fd[NF], qd[3] = {q[0], q[1], q[2]}, ed;
