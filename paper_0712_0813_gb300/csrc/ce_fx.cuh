@@ -128,21 +128,6 @@ CE_FX_HD double to_double(const Fx& x) {
   return from_bits((s & INT64_MIN) | (e << 52) | (frac & 0xfffffffffffffLL));
 }
 
-// r 2^u as a double, to nearest; 0 below the normal range.  RANGE: infinite above
-// it (else the caller knows that r 2^u stays clear of that).
-template <bool RANGE>
-CE_FX_HD double scaled(int64_t r, int u) {
-  const int64_t s = r >> 63;
-  uint64_t a = (uint64_t)((r ^ s) - s);
-  const int z = clz64(a);
-  a <<= z & 63;
-  const int eb = u - z + 63 + 1023;
-  int64_t b = (int64_t)((a >> 11) + ((a >> 10) & 1)) + ((int64_t)(eb - 1) << 52);
-  if (RANGE) b = eb >= kNonFinite ? 0x7ff0000000000000LL : b;
-  b = (eb < 1 || z == 64) ? 0 : b;
-  return from_bits(b | (s & INT64_MIN));
-}
-
 // x >> s of an unsigned value, s >= 0 of any size.
 CE_FX_HD uint64_t lsr(uint64_t x, int s) {
 #ifdef __CUDA_ARCH__
@@ -152,6 +137,25 @@ CE_FX_HD uint64_t lsr(uint64_t x, int s) {
 #else
   return s > 63 ? 0 : x >> s;
 #endif
+}
+
+// (x >> s) of an unsigned value, to nearest, for s >= 1.
+CE_FX_HD int64_t lsr_round(uint64_t x, int s) { return (int64_t)((lsr(x, s - 1) + 1) >> 1); }
+
+// r 2^u as a double, to nearest, subnormal below the normal range.  RANGE: infinite
+// above it (else the caller knows that r 2^u stays clear of that).
+template <bool RANGE>
+CE_FX_HD double scaled(int64_t r, int u) {
+  const int64_t s = r >> 63;
+  uint64_t a = (uint64_t)((r ^ s) - s);
+  const int z = clz64(a);
+  a <<= z & 63;
+  const int eb = u - z + 63 + 1023;
+  int64_t b = (int64_t)((a >> 11) + ((a >> 10) & 1)) + ((int64_t)(eb - 1) << 52);
+  if (RANGE) b = eb >= kNonFinite ? 0x7ff0000000000000LL : b;
+  b = z == 64 ? 0 : b;
+  if (eb < 1) b = lsr_round(a, 12 - eb);   // in units of 2^-1074
+  return from_bits(b | (s & INT64_MIN));
 }
 
 // The upper 64 bits of a product: the product of two 64-bit fractions.
@@ -243,9 +247,6 @@ CE_FX_HD bool fast_site(const int (&em)[NF], const SiteModel<NF>& s) {
   for (int i = 0; i < NF; ++i) ok = ok && em[i] < 1023 + 200 && s.ud[i] + 2 < em[i] - kOne;
   return ok;
 }
-
-// (x >> s) of an unsigned value, to nearest, for s >= 1.
-CE_FX_HD int64_t lsr_round(uint64_t x, int s) { return (int64_t)((lsr(x, s - 1) + 1) >> 1); }
 
 // A site's force over 1/dx^2 and its term of the energy sum that drives a(t).
 //   force[i] = raw_i - dx^2 dV/df_i, raw_i = sum of the 2d neighbours - 2d g_i
