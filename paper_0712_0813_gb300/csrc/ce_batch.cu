@@ -88,7 +88,7 @@ __device__ __forceinline__ double member_source(const BMember<float>* m, float g
   return block_source(g2, 0.f, pot, 0.f, m->source);
 }
 __device__ __forceinline__ double member_source(const BMember<double>* m, double g2, double pot) {
-  return block_sum(fma(pot, (double)m->source.ratio + (double)m->source.ratio_lo, g2)) * m->source.weight;
+  return block_sum(fma(pot, m->source.wv, g2 * m->source.wg));
 }
 
 struct BItem {

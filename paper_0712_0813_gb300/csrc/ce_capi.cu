@@ -51,17 +51,6 @@ constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz: bound of ever
 
 void ce::set_last_error(const std::string& msg) { g_err = msg; }
 
-// 2 G + 3 V = <(df)^2> / dx^2 + 3 <V> with G = <(df)^2> / (2 dx^2).
-ce::SourceWeights ce::source_weights(double dx, int64_t S) {
-  const double ratio = 3.0 * dx * dx;
-  SourceWeights w;
-  w.weight = 1.0 / (dx * dx * (double)S);
-  w.ratio = (float)ratio;
-  w.ratio_lo = (float)(ratio - (double)w.ratio);
-  return w;
-}
-
-
 namespace {
 
 void* dalloc(ce_sim* s, size_t n) {

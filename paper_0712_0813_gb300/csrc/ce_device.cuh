@@ -172,7 +172,8 @@ __device__ __forceinline__ void warp_sum_pair(FloatPair& x) {
 // A block's share of 2 G + 3 V from its threads' two-level FP32 sums g0 + g1 and
 // v0 + v1 (fixed order, valid in thread 0).  The sums are combined and added as float
 // pairs (the per-thread sums' own rounding stays what limits them): three FP64
-// instructions a block; sums that would leave FP32's range take FP64 throughout.
+// instructions a block; sums that would leave the range in which a pair holds 48 bits
+// of them, or of their products, take FP64 throughout.
 __device__ __forceinline__ double block_source(float g0, float g1, float v0, float v1, const SourceWeights& k) {
   __shared__ float2 part[32];
   __shared__ double wide[32];
@@ -184,24 +185,25 @@ __device__ __forceinline__ double block_source(float g0, float g1, float v0, flo
   const float p = __fmul_rn(k.ratio, v.hi);
   t.lo += fmaf(k.ratio, v.hi, -p) + fmaf(k.ratio_lo, v.hi, k.ratio * v.lo);
   add_to(t.hi, t.lo, p);
-  const bool fits = fabsf(t.hi) < 1e32f;
+  const float size = fabsf(t.hi);
+  const bool fits = size < 0x1p100f && (size > 0x1p-90f || (t.hi == 0.f && v.hi == 0.f));
   warp_sum_pair<32>(t);
   if (lane == 0) part[warp] = make_float2(t.hi, t.lo);
   if (__syncthreads_or(!fits)) {
-    const double q = warp_sum(fma((double)v0 + (double)v1, (double)k.ratio + (double)k.ratio_lo, (double)g0 + (double)g1));
+    const double q = warp_sum(fma((double)v0 + (double)v1, k.wv, ((double)g0 + (double)g1) * k.wg));
     if (lane == 0) wide[warp] = q;
     __syncthreads();
     double sum = 0.0;
     if (threadIdx.x == 0)
       for (int w = 0; w < nwarps; ++w) sum += wide[w];
-    return sum * k.weight;
+    return sum;
   }
   double q = 0.0;
   if (warp == 0) {
     const float2 x = lane < nwarps ? part[lane] : make_float2(0.f, 0.f);
     FloatPair s{x.x, x.y};
     warp_sum_pair<32>(s);
-    if (lane == 0) q = ((double)s.hi + (double)s.lo) * k.weight;
+    if (lane == 0) q = ((double)s.hi + (double)s.lo) * k.wg;
   }
   return q;
 }
@@ -308,8 +310,7 @@ __device__ __forceinline__ void finish_step_sums(const StepArgs<float>& p, float
 }
 // And from FP64 sums.
 __device__ __forceinline__ void finish_step_sums(const StepArgs<double>& p, double g0, double g1, double v0, double v1) {
-  const double ratio = (double)p.source.ratio + (double)p.source.ratio_lo;
-  finish_step(p, block_sum(fma(v0 + v1, ratio, g0 + g1)) * p.source.weight);
+  finish_step(p, block_sum(fma(v0 + v1, p.source.wv, (g0 + g1) * p.source.wg)));
 }
 
 }  // namespace ce

@@ -49,7 +49,7 @@ __device__ __forceinline__ Fx shfl_down(const Fx& x) {
 
 // End of a step from the threads' energy terms: 2 G + 3 V = -dx^-2 <energy>.
 __device__ __forceinline__ void finish(const StepArgs<double>& p, double energy) {
-  finish_step(p, block_sum(energy) * -p.source.weight);
+  finish_step(p, block_sum(energy) * -p.source.wg);
 }
 
 // ---- 3D ---------------------------------------------------------------------

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "ce_fx.cuh"
+#include "ce_source.h"
 #include "clusterlat.h"
 
 namespace ce {
@@ -54,15 +55,6 @@ struct DevAux {
   int pad;
   double result[kResultLen];
 };
-
-// How a block's sums enter the source 2 G + 3 V of the scale factor: weight times
-// (sum of (df)^2 + ratio times sum of V), the ratio 3 dx^2 as a float pair.
-struct SourceWeights {
-  double weight;
-  float ratio, ratio_lo;
-};
-
-SourceWeights source_weights(double dx, int64_t S);
 
 // Arguments of one step launch.  T is the storage/arithmetic type of fields
 // and velocities; the global sums and scalars are always double.

@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(Shape<T>::threads, 1) k_resident(const Residen
     double share = 0.0;
     if constexpr (!SUMS) __syncthreads();
     else if constexpr (sizeof(T) == 4) share = block_source(g0, g1, v0, v1, p.source);
-    else share = block_sum(g0) * p.source.weight;
+    else share = block_sum(g0) * p.source.wg;
     if (tid == 0) {
       if (SUMS) __stcg(p.shares + (size_t)(step & 1) * blocks + blockIdx.x, share);
       arrive(p.counter);   // releases the block's stores, ordered before by the barrier
