@@ -63,8 +63,8 @@ WORKLOAD = WORKLOADS["1024cube"]
 METRIC = "Gsite-updates/s"
 GOLDEN_256 = os.path.join(ROOT, "tests", "golden", "longrun_256cube.json")
 STEP_SOURCES = {"k_step_sweep": ("ce_sweep3d.cuh", "ce_sweep3d_f32.cu", "ce_tma.cuh", "ce_device.cuh",
-                                 "ce_internal.h"),
-                "k_step_generic": ("ce_generic.cu", "ce_device.cuh", "ce_internal.h")}
+                                 "ce_internal.h", "ce_source.h"),
+                "k_step_generic": ("ce_generic.cu", "ce_device.cuh", "ce_internal.h", "ce_source.h")}
 
 
 def dist_env():

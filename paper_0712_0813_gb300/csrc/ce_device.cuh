@@ -56,10 +56,6 @@ __device__ __forceinline__ T ldg_at(const T* base, uint32_t bytes) {
   return __ldg(reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + bytes));
 }
 template <typename T>
-__device__ __forceinline__ void st_at(T* base, uint32_t bytes, T v) {
-  *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + bytes) = v;
-}
-template <typename T>
 __device__ __forceinline__ void stcs_at(T* base, uint32_t bytes, T v) {
   __stcs(reinterpret_cast<T*>(reinterpret_cast<char*>(base) + bytes), v);
 }
@@ -223,55 +219,10 @@ __device__ __forceinline__ double block_sum(double a) {
   return a;
 }
 
-// Scale-factor update of reading c-4, done once per step by one thread:
-//   a_{n+1} = a_n + dt a'_{n+1/2}
-//   Q = kappa2 (2 G + 3 V) / a_{n+1},  C = 2 a'_{n+1/2} + dt Q
-//   u = a'_{n+3/2} + a'_{n+1/2} = 2 C / (1 + sqrt(1 + dt C / a_{n+1}))
-// (closed form of the implicit midpoint a'_new - a'_old = dt (-(u/2)^2/a + Q)),
-//   a''_{n+1} = (u - 2 a'_{n+1/2}) / dt,  a'_{n+3/2} = u - a'_{n+1/2}.
-// In two parts: what does not need the sums (scale_ahead) can run before they are
-// there.  y = u / C solves (e/4) y^2 + y = 1 with e = dt C / a: for small e two
-// Newton steps in FP64 with FP32's slope, from FP32's root (errors 1e-7, 1e-14, 0),
-// are six instructions where the square root and the division take eighteen.
-struct ScaleAhead {
-  double a, ap, ap2, ia, dia, k1, e1;
-};
-__device__ __forceinline__ ScaleAhead scale_ahead(const DevScalars& in, double dt, double kappa2) {
-  ScaleAhead s;
-  s.a = fma(dt, in.ap, in.a);
-  s.ap = in.ap;
-  s.ap2 = in.ap + in.ap;
-  s.ia = 1.0 / s.a;
-  s.dia = dt * s.ia;
-  s.k1 = kappa2 * s.dia;
-  s.e1 = 0.25 * s.dia;
-  return s;
-}
-// source: 2 G + 3 V.
+// The update (ce_source.h) by one thread; a source that leaves no real a' is latched.
 __device__ __forceinline__ void scale_factor_update(const ScaleAhead& s, DevScalars& out, double source, double inv_dt,
                                                     int* status) {
-  const double C = fma(s.k1, source, s.ap2);
-  const double e4 = s.e1 * C;
-  const float e = 4.f * (float)e4;
-  double y;
-  if (fabsf(e) < 0.25f) {
-    const float yf = 2.f / (1.f + sqrtf(1.f + e));
-    const double slope = (double)(1.f / (1.f + 0.5f * e * yf));
-    y = (double)yf;
-    y = fma(fma(-(e4 * y), y, 1.0 - y), slope, y);
-    y = fma(fma(-(e4 * y), y, 1.0 - y), slope, y);
-  } else {   // also where something is not finite
-    const double disc = fma(4.0, e4, 1.0);
-    if (!(disc >= 0.0) || !isfinite(source)) atomicCAS(status, CE_OK, CE_ENONFINITE);
-    y = 2.0 / (1.0 + sqrt(disc));
-  }
-  const double u = C * y;
-  const double app = (u - s.ap2) * inv_dt;
-  out.c = app * s.dia;
-  out.app = app;
-  out.s = app * s.ia;
-  out.a = s.a;
-  out.ap = u - s.ap;
+  if (!scale_update(s, out, source, inv_dt)) atomicCAS(status, CE_OK, CE_ENONFINITE);
 }
 
 // End of a step launch: publish this block's share of 2 G + 3 V (in thread 0), and

@@ -14,22 +14,6 @@
 
 namespace ce {
 
-// Scale-factor state belonging to one integer time t_n.  Two slots alternate
-// between step launches (launch k reads slot k%2 and writes slot (k+1)%2), so a
-// launch never overwrites what its own blocks are still reading.
-//
-// The velocity state kept in HBM is w with  f'(t_n + dt/2) = w + c f(t_n).  The
-// fused step kernel cannot add the expansion term (a''/a) f of its own kick,
-// because a'' needs the global sums of the f it is writing; that term is folded
-// in by the next launch through c = dt a''/a (and c = 0 after a restore).
-struct DevScalars {
-  double a;    // a(t_n)
-  double ap;   // a'(t_n + dt/2)
-  double app;  // a''(t_n)
-  double s;    // a''(t_n) / a(t_n)
-  double c;    // coefficient of f in the velocity reconstruction above
-};
-
 constexpr int kResultLen = 64;
 
 // Result layout of the diagnostics pass (doubles).
@@ -78,7 +62,7 @@ struct StepArgs {
   int update_scalars;   // 1: reduce G, V and advance a, a', a'' in the last block
   int in_slot;          // which ping-pong buffer set is the input (selects TMA maps)
   long long wait_cycles;      // bound of every mbarrier wait (SM clock cycles)
-  unsigned int missing_tx;    // test-only: bytes announced per plane that never arrive
+  unsigned int missing_tx;    // test-only: bytes a plane (z-sweep kernel) or arrivals a barrier (3D FP64 kernel) waits for in vain
   const DevScalars* sc_in;
   DevScalars* sc_out;
   double* partials;     // one per block
