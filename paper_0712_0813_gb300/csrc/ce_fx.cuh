@@ -105,6 +105,14 @@ CE_FX_HD int clz64(uint64_t x) {
 #endif
 }
 
+CE_FX_HD int clz32(int x) {
+#ifdef __CUDA_ARCH__
+  return __clz(x);
+#else
+  return x ? __builtin_clz((unsigned)x) : 32;
+#endif
+}
+
 CE_FX_HD int imax(int a, int b) { return a > b ? a : b; }
 CE_FX_HD int imin(int a, int b) { return a < b ? a : b; }
 
@@ -277,7 +285,13 @@ CE_FX_HD void site_force(const Fx (&g)[NF], const Fx (&nb)[NF][2 * DIMS], const 
     for (int j = 0; j < 2 * DIMS; ++j) raw += asr(nb[i][j].m, em[i] - nb[i][j].e);
     const int ur = em[i] - kOne;
     // |raw| <= 3 2^60: at least two leading bits free (zero: as far as the model force likes)
-    const int up = imin(raw == 0 ? 8192 : clz64((uint64_t)(raw ^ (raw >> 63))) - 2, ur - s.ud[i] - 2);
+    const int rs = (int)(raw >> 63), rh = (int)(raw >> 32) ^ rs;
+    int lead = clz32(rh);
+    if (rh == 0) {
+      const int rl = (int)raw ^ rs;
+      lead = rl == 0 && rs == 0 ? 8192 : 32 + clz32(rl);
+    }
+    const int up = imin(lead - 2, ur - s.ud[i] - 2);
     int u;
     if constexpr (FAST) {
       raw = shl(raw, up);
