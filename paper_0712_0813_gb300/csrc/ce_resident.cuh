@@ -53,6 +53,7 @@ constexpr int64_t max_sites(int dims, int nf) {
   return nf <= 2 ? (dims == 3 ? 900000 : 1100000) : (dims == 3 ? 600000 : 700000);
 }
 
+constexpr size_t kStaticSmem = 8192;   // room left for the kernel's static shared memory
 constexpr int kHeld = 2;   // halo sites a thread holds in registers while a' is formed
 
 // Consecutive sites of which a thread adds the energy terms in T before they join its
@@ -441,6 +442,7 @@ ResidentPlan plan(int dims, int64_t N, int nf, int device, int sms) {
     return pl;
   }
   const int n = (int)N;
+  const size_t room = (size_t)limit - kStaticSmem;
   int64_t best = INT64_MAX;
   for (int nz = 1; nz <= (dims == 3 ? std::min(n, sms) : 1); ++nz)
     for (int ny = 1; ny <= (dims >= 2 ? std::min(n, sms / nz) : 1); ++ny)
@@ -453,7 +455,7 @@ ResidentPlan plan(int dims, int64_t N, int nf, int device, int sms) {
         const int64_t padded = (int64_t)(bx + 2) * (dims >= 2 ? by + 2 : 1) * (dims == 3 ? bz + 2 : 1);
         if (padded > 65535) continue;
         const size_t bytes = smem_bytes<T>(nf, (int)padded, (int)sites, (int)halo);
-        if (bytes + 8192 > (size_t)limit) continue;   // the kernel's static shared memory
+        if (bytes > room) continue;
         if (sites + halo < best) {
           best = sites + halo;
           pl = ResidentPlan{bx, by, bz, nx, ny, nz, nx * ny * nz, 0, (int)bytes};
@@ -465,7 +467,8 @@ ResidentPlan plan(int dims, int64_t N, int nf, int device, int sms) {
   for (int sums = 0; sums < 2; ++sums) {
     const void* k = kernel<T>(nf, dims, sums != 0);
     int per_sm = 0;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.smem) != cudaSuccess ||
+    // one value for every lattice: the attribute is the kernel's, not the handle's
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, pl.threads, pl.smem) != cudaSuccess || per_sm < 1) {
       cudaGetLastError();
       return ResidentPlan{};
