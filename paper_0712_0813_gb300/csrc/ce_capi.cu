@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "ce_internal.h"
+#include "ce_plan.h"
 #include "clusterlat.h"
 
 namespace {
@@ -520,7 +521,8 @@ int ce_create(const ce_config* cfg, ce_sim** out) {
   // read from fluctuations of 1e-2 about 1 and show the difference (up to 3e-4 after
   // 1000 steps; with more fields below 1e-6).
   const bool rounding_shows = s->prec == CE_F32 && s->nf == 1 && s->cfg.expansion;
-  if (cfg->kernel == CE_KERNEL_AUTO && !sweep_hinted && !rounding_shows && !(cfg->flags & CE_FLAG_TEST_TMA_STALL)) {
+  if (cfg->kernel == CE_KERNEL_AUTO && !sweep_hinted && !rounding_shows && !(cfg->flags & CE_FLAG_TEST_TMA_STALL) &&
+      ce::plan::resident_takes(s->dims, S, s->nf, s->prec == CE_F64, s->cfg.expansion != 0)) {
     s->res = s->prec == CE_F32 ? ce::resident_plan_f32(s->dims, s->N, s->nf, s->device, s->sms)
                                : ce::resident_plan_f64(s->dims, s->N, s->nf, s->device, s->sms);
     if (s->res.blocks > 0) {

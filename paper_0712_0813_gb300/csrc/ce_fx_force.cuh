@@ -30,9 +30,10 @@ static __device__ __noinline__ void force_fp64(const double* g, const double* nb
   *energy = DIMS == 1 ? fma(-3.0 * dx2, vs, e) : e;
 }
 
-// The site's force by the form its values allow.  In 1D the energy term is that of
+// The site's force by the form its values allow; GENERAL leaves the fast form out, for
+// kernels whose code is long enough without it.  In 1D the energy term is that of
 // line_energy, with its sign turned.
-template <int NF, int DIMS, bool SUMS>
+template <int NF, int DIMS, bool SUMS, bool GENERAL = false>
 __device__ __forceinline__ void force_of(const Fx (&g)[NF], const Fx (&nb)[NF][2 * DIMS], const FxModel& k,
                                          double inv_dx2, const double (&q)[3], double (&force)[NF], double& energy) {
   const int flip = -(int)(threadIdx.x & 1u);
@@ -44,7 +45,7 @@ __device__ __forceinline__ void force_of(const Fx (&g)[NF], const Fx (&nb)[NF][2
 #pragma unroll
   for (int i = 0; i < NF; ++i) up[i] = nb[i][1];
   constexpr bool kParts = SUMS && DIMS > 1;
-  if (fast_site<NF>(em, s)) {
+  if (!GENERAL && fast_site<NF>(em, s)) {
     site_force<NF, DIMS, kParts, true>(g, nb, em, s, flip, force, energy);
     if constexpr (SUMS && DIMS == 1) energy = -line_energy<NF>(g, up, s);
     return;

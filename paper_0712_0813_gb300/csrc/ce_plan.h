@@ -193,5 +193,31 @@ inline int wave_chunk_length(int64_t N, int64_t blocks_per_chunk, int64_t slots,
   return (int)best_len;
 }
 
+// Whether a lattice takes the resident kernel (many steps in one cooperative launch,
+// ce_resident.cuh) on the automatic choice: where a handle that has the GPU to itself
+// steps clearly faster than with one launch a step, calls of one step are no slower
+// than they were without the resident kernel, and 16 handles on streams of their own are not
+// slower by more than that gains.  us a step of two fields, resident against one launch
+// a step, one handle / 16 at once (and, in brackets, in calls of one step):
+//   FP32, expanding: 3D 32^3 4.8 / 0.83 against 9.3 / 0.84, 48^3 5.4 / 2.0 against 8.8 /
+//     1.2, 64^3 7.0 / 4.7 (14.4) against 9.7 / 3.0 (11.6), 80^3 10.9 / 8.6 against 9.6 /
+//     4.7; four fields 48^3 6.9 / 3.4 against 9.6 / 2.4, 64^3 10.4 / 7.8 (18.5) against
+//     11.5 / 6.0 (14.4); 2D 600^2 6.6 / 4.0 against 11.5 / 4.5, 1000^2 9.4 / 9.7 (18.5)
+//     against 15.0 / 8.9 (16.6); 1D 131072 4.9 / 1.5 against 6.3 / 0.8, 300000 6.2 / 2.3
+//     (14.4) against 6.7 / 2.0 (8.3).
+//   FP32, no expansion: no sum ends a step there, and the launches of a graph follow
+//     each other in 2 to 5 us.  3D 20^3 1.9 / 0.39 against 5.0 / 0.51, 32^3 2.6 / 0.60
+//     against 5.0 / 0.58, 40^3 3.7 / 0.89 against 5.0 / 0.71; 2D 200^2 2.4 (6.3) against
+//     2.7 (4.2), 600^2 and above, where the row kernel is the other one, 3.6 / 2.6
+//     against 7.0 / 3.8, 800^2 5.3 (12.4) against 9.3 (11.6).
+//   FP64: 3D 40^3 8.0 / 5.1 against 12.8 / 5.3, 72^3 21 against 25; 2D 700^2 21 against 23;
+//     1D 590000 22 against 23.  The shared memory of a block per SM ends little above that.
+inline bool resident_takes(int dims, int64_t S, int nf, bool f64, bool expansion) {
+  if (f64) return S <= (dims == 3 ? 450000 : 600000);
+  if (!expansion) return dims == 3 ? S * nf <= 65536 : dims == 2 && S >= 360000 && S <= 700000;
+  if (dims == 1) return S <= 150000;
+  return S * nf <= (dims == 3 ? 524288 : 2000000);
+}
+
 }  // namespace plan
 }  // namespace ce

@@ -30,27 +30,33 @@
 namespace ce {
 namespace resident {
 
-template <typename T>
-struct Shape;
-template <>
-struct Shape<float> {
-  static constexpr int threads = 1024;     // most threads of a block
-};
-template <>
-struct Shape<double> {
-  static constexpr int threads = 512;
+// Most threads of a block, and resident blocks per SM the registers are bounded for.
+// FP64 with three and four fields spilt at 512 threads (four at 33^3: 13.3 us a step,
+// 11.9 at 384, two dimensions at 400^2 16.9 and 15.6).
+template <typename T, int NF>
+struct Shape {
+  static constexpr int threads = sizeof(T) == 8 && NF > 2 ? 384 : 512;
+  static constexpr int blocks = sizeof(T) == 8 ? 1 : 2;
 };
 
-// Lattices up to this many sites take the resident kernel, where it was found faster
-// than one launch a step (us a step, two fields, expanding; resident against the best
-// other): FP32 3D 64^3 7.4 / 12, 96^3 11.9 / 15.8, 100^3 13.9 / 13.3; 2D 1000^2 9.3 /
-// 14.7; 1D 1.1 M 7.6 / 19.9; four fields 80^3 14.7 / 16.0, 88^3 14.6 / 14.5; FP64
-// 64^3 15.5 / 21.4, 72^3 19.7 / 23.9, 80^3 26.3 / 25.9; 2D 700^2 19.2 / 21.7; 1D 590000
-// 19.6 / 21.6.  The shared memory of one block per SM ends little above that.
+// Blocks and threads.  A block per SM and a thread per site would be the shortest step
+// of a lattice that has the GPU to itself, but not by much: half the SMs serve small
+// lattices as well (fewer blocks in the exchange), and two to four sites a thread hide
+// their own latency.  What is left free lets other handles' launches run beside this
+// one.  us a step, two fields, expanding, one handle / 16 handles on their own streams,
+// with a thread per site on every SM and as below: FP32 20^3 4.2 / 0.75 and 3.9 / 0.52,
+// 32^3 4.3 / 1.55 and 4.8 / 0.83, 48^3 5.6 / 5.6 and 5.4 / 2.0, 64^3 7.4 / 7.3 and
+// 7.0 / 4.6; 2D 300^2 4.9 / 4.9 and 4.9 / 1.5, 700^2 7.7 / 7.6 and 7.2 / 4.4; FP64 16^3
+// 5.5 / 1.4 and 5.5 / 0.76, 48^3 10.2 / 10.2 and 10.1 / 6.9, 1D 65536 7.3 / 7.3 and
+// 7.1 / 4.1.
 template <typename T>
-constexpr int64_t max_sites(int dims, int nf) {
-  if (sizeof(T) == 8) return dims == 3 ? 450000 : 600000;
-  return nf <= 2 ? (dims == 3 ? 900000 : 1100000) : (dims == 3 ? 600000 : 700000);
+int blocks_limit(int64_t S, int sms) {
+  return S <= (sizeof(T) == 4 ? 70000 : 12000) ? std::max(1, sms / 2) : sms;
+}
+template <typename T>
+int threads_limit(int dims, int nf, int64_t sites, int64_t halo) {
+  if (sizeof(T) == 4) return sites + halo <= (dims == 3 ? 1500 : 2500) ? 256 : 512;
+  return sites * nf <= 2000 ? 256 : (nf > 2 ? Shape<T, 4>::threads : Shape<T, 2>::threads);
 }
 
 constexpr size_t kStaticSmem = 8192;   // room left for the kernel's static shared memory
@@ -209,7 +215,7 @@ __device__ __forceinline__ void kick(const ResidentArgs<double>& p, const Tile<d
   }
   double force[NF], energy;
   const double q[3] = {p.q[0], p.q[1], p.q[2]};
-  fx::force_of<NF, DIMS, SUMS>(g, nb, p.model, p.inv_dx2, q, force, energy);
+  fx::force_of<NF, DIMS, SUMS, (NF > 3)>(g, nb, p.model, p.inv_dx2, q, force, energy);
   if (SUMS) s0 -= energy;
   const double kk = p.dt * p.inv_dx2;
 #pragma unroll
@@ -233,7 +239,7 @@ __device__ __forceinline__ bool wait_for(unsigned* counter, unsigned want, long 
 }
 
 template <typename T, int NF, int DIMS, bool SUMS>
-__global__ void __launch_bounds__(Shape<T>::threads, 1) k_resident(const ResidentArgs<T> p) {
+__global__ void __launch_bounds__(Shape<T, NF>::threads, Shape<T, NF>::blocks) k_resident(const ResidentArgs<T> p) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ DevScalars s_sc;
   __shared__ int s_abort;
@@ -408,9 +414,12 @@ __global__ void __launch_bounds__(Shape<T>::threads, 1) k_resident(const Residen
   if (tid == 0 && s_abort) atomicCAS(p.status, CE_OK, CE_ETIMEOUT);
 }
 
+// Null where no lattice takes it (plan::resident_takes).
 template <typename T, int NF, int DIMS>
 const void* kernel_of(bool sums) {
-  return sums ? (const void*)k_resident<T, NF, DIMS, true> : (const void*)k_resident<T, NF, DIMS, false>;
+  if (sums) return (const void*)k_resident<T, NF, DIMS, true>;
+  if constexpr (sizeof(T) == 8 || DIMS >= 2) return (const void*)k_resident<T, NF, DIMS, false>;
+  return nullptr;
 }
 template <typename T, int NF>
 const void* kernel_dims(int dims, bool sums) {
@@ -428,13 +437,13 @@ const void* kernel(int nf, int dims, bool sums) {
 
 // The bricks of a lattice: counts per axis with at most one block per SM, the
 // least sites plus halo in the largest brick; none where a brick does not fit the
-// shared memory or the lattice is larger than what the kernel was found faster for.
+// shared memory.
 template <typename T>
 ResidentPlan plan(int dims, int64_t N, int nf, int device, int sms) {
   ResidentPlan pl{};
   int64_t S = 1;
   for (int d = 0; d < dims; ++d) S *= N;
-  if (S > max_sites<T>(dims, nf)) return pl;
+  sms = blocks_limit<T>(S, sms);
   int coop = 0, limit = 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess || !coop ||
       cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) {
@@ -459,13 +468,14 @@ ResidentPlan plan(int dims, int64_t N, int nf, int device, int sms) {
         if (sites + halo < best) {
           best = sites + halo;
           pl = ResidentPlan{bx, by, bz, nx, ny, nz, nx * ny * nz, 0, (int)bytes};
-          const int per = (int)std::min<int64_t>((sites / g + 31) / 32 * 32, Shape<T>::threads);
+          const int per = (int)std::min<int64_t>((sites / g + 31) / 32 * 32, threads_limit<T>(dims, nf, sites, halo));
           pl.threads = std::max(per, 128);
         }
       }
   if (pl.blocks == 0) return pl;
   for (int sums = 0; sums < 2; ++sums) {
     const void* k = kernel<T>(nf, dims, sums != 0);
+    if (!k) continue;
     int per_sm = 0;
     // one value for every lattice: the attribute is the kernel's, not the handle's
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room) != cudaSuccess ||
