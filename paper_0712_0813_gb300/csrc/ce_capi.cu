@@ -4,6 +4,7 @@
 // in the kernels; this file only moves data and sequences launches.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -152,16 +153,30 @@ ce::StepArgs<T> make_step_args(const ce_sim* s, int in, bool half_kick) {
   return a;
 }
 
+// The integer force is formed in units of 1/dx^2, so dx^2 times the model force has to
+// stay in FP64's range: spacings above 2^200 count as that, where the Laplacian (below
+// 2^-396 of the fields) is lost beside anything else either way.
+template <typename Args>
+void fx_spacing(const ce_sim* s, Args& a) {
+  const double dx = std::min(s->dx, 0x1p200);
+  a.inv_dx2 = 1.0 / (dx * dx);
+  a.source = ce::source_weights(dx, s->S);
+}
+
 template <typename T>
 cudaError_t launch_one_step(const ce_sim* s, int in, bool half_kick) {
   if (s->kernel == CE_KERNEL_ROWS && !half_kick) return ce::rows_launch(s->rows, in, s->stream);
-  const ce::StepArgs<T> a = make_step_args<T>(s, in, half_kick);
+  ce::StepArgs<T> a = make_step_args<T>(s, in, half_kick);
   if (s->kernel == CE_KERNEL_SWEEP) return ce::launch_step_sweep<T>(a, s->plan, s->stream);
   if (s->kernel == CE_KERNEL_PLANES)
     return s->dims == 3 ? ce::launch_step_cols<T>(a, s->cols, s->stream)
                         : ce::launch_step_lines<T>(a, s->lines, s->stream);
-  if constexpr (sizeof(T) == 8) return ce::launch_step_fx(a, s->fx, s->stream);
-  else return ce::launch_step_generic(a, s->generic_blocks, s->stream);
+  if constexpr (sizeof(T) == 8) {
+    fx_spacing(s, a);
+    return ce::launch_step_fx(a, s->fx, s->stream);
+  } else {
+    return ce::launch_step_generic(a, s->generic_blocks, s->stream);
+  }
 }
 
 cudaError_t step_once(const ce_sim* s, int in, bool half_kick) {
@@ -190,7 +205,10 @@ cudaError_t launch_resident_steps(ce_sim* s, int in, int n) {
   a.inv_ddt = 1.0 / s->cfg.dt;
   a.kappa2 = s->kappa2;
   a.source = ce::source_weights(s->dx, s->S);
-  if constexpr (sizeof(T) == 8) a.model = ce::fx_model(a.dt, a.inv_dx2, s->cfg.q);
+  if constexpr (sizeof(T) == 8) {
+    fx_spacing(s, a);
+    a.model = ce::fx_model(a.dt, a.inv_dx2, s->cfg.q);
+  }
   a.slot = s->aux->slot;
   a.counter = s->res_counter;
   a.count0 = s->res_count;
