@@ -72,9 +72,26 @@ extern "C" {
 #define CE_KERNEL_AUTO    0 /* FP32: z-sweep kernel where it applies; else the
                                row kernel for 2D sides >= 512 and 3D sides >= 256
                                it takes; else the column kernel (3D) or the
-                               line-sweep kernel (2D sides >= 320); else generic.  FP64: generic (the force in
-                               integer arithmetic), or the z-sweep kernel when plan hints
-                               (tile_rows, stages, zchunks) are given          */
+                               line-sweep kernel (2D sides >= 320); else generic.
+                               FP64: generic (the force in integer arithmetic),
+                               or the z-sweep kernel when plan hints (tile_rows,
+                               stages, zchunks) are given.
+                               Small lattices, without plan hints: ce_step takes
+                               the resident kernel instead, up to 4096 steps in
+                               one cooperative launch with up to a block on every
+                               SM.  FP64: to 450000 sites in 3D, 600000 else.
+                               FP32 with expansion and two fields or more: sites
+                               x fields to 524288 in 3D, 2000000 in 2D, 150000
+                               sites in 1D.  FP32 without expansion: sites x
+                               fields to 65536 in 3D, 360000 to 700000 sites in
+                               2D.  One handle at a time is what it is fastest
+                               for: four and more FP32 handles of 41^3 to 64^3
+                               sites stepped at once on streams of their own run
+                               up to 1.6 times faster with CE_KERNEL_PLANES, and
+                               a batch is faster than either.  Steps that the
+                               caller captures into a graph of its own, and
+                               handles on a stream that may use part of the GPU
+                               only, take one launch a step                    */
 #define CE_KERNEL_GENERIC 1 /* any d and N: one thread per site (FP32), strips of
                                30 sites with the force in integers (FP64)      */
 #define CE_KERNEL_SWEEP   2 /* 3D z-sweep kernel (CE_EINVAL if it does not apply) */
@@ -223,8 +240,14 @@ const char* ce_last_error(void);
 /* Bytes of device memory the handle holds (state + scratch). */
 int64_t ce_device_bytes(const ce_sim* sim);
 
-/* Which kernel ce_step launches: CE_KERNEL_GENERIC, _SWEEP, _ROWS or _PLANES. */
+/* Which kernel advances the handle where a step is one launch (and in the
+ * start-up): CE_KERNEL_GENERIC, _SWEEP, _ROWS or _PLANES. */
 int ce_kernel_in_use(const ce_sim* sim);
+
+/* 1 if ce_step advances the handle by the resident kernel (CE_KERNEL_AUTO), 0 if
+ * by one launch of ce_kernel_in_use a step (also after its stream turned out not
+ * to take the resident kernel's cooperative launch). */
+int ce_resident_in_use(const ce_sim* sim);
 
 /* The z-sweep launch plan in use: tile rows, pipeline stages and z-chunks
  * (all 0 when the generic kernel runs).  Errors: CE_EINVAL (NULL argument). */

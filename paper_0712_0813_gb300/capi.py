@@ -60,7 +60,7 @@ _keepalive: dict = {}   # handle -> (config, ctypes callbacks, allocation table)
 # Every symbol the public header declares (checked by the test-suite).
 EXPORTS = ("ce_create", "ce_set_fields", "ce_step", "ce_synchronize", "ce_means_variances",
            "ce_energy", "ce_get_fields", "ce_free", "ce_last_error", "ce_device_bytes",
-           "ce_kernel_in_use", "ce_sweep_plan", "ce_replan", "ce_version", "ce_moments_noalloc",
+           "ce_kernel_in_use", "ce_resident_in_use", "ce_sweep_plan", "ce_replan", "ce_version", "ce_moments_noalloc",
            "ce_spectrum", "ce_save", "ce_load",
            "ce_sample_fields", "ce_batch_create", "ce_batch_step", "ce_batch_synchronize", "ce_batch_status", "ce_batch_info",
            "ce_batch_free")
@@ -95,6 +95,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
         "ce_last_error": (ctypes.c_char_p, []),
         "ce_device_bytes": (ctypes.c_int64, [vp]),
         "ce_kernel_in_use": (ctypes.c_int, [vp]),
+        "ce_resident_in_use": (ctypes.c_int, [vp]),
         "ce_sweep_plan": (ctypes.c_int, [vp, P(ctypes.c_int), P(ctypes.c_int), P(ctypes.c_int)]),
         "ce_replan": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
         "ce_spectrum": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_int, pd, pd, pd]),
@@ -255,6 +256,10 @@ def ce_kernel_in_use(sim) -> int:
     return load().ce_kernel_in_use(sim)
 
 
+def ce_resident_in_use(sim) -> int:
+    return load().ce_resident_in_use(sim)
+
+
 def ce_sweep_plan(sim):
     """(rows, stages, zchunks) of the z-sweep plan; zeros when the generic kernel runs."""
     r, st, z = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
@@ -405,6 +410,10 @@ class Simulation:
     @property
     def kernel(self):
         return ce_kernel_in_use(self.handle)
+
+    @property
+    def resident(self) -> bool:
+        return bool(ce_resident_in_use(self.handle))
 
     @property
     def sweep_plan(self):

@@ -793,6 +793,8 @@ int64_t ce_device_bytes(const ce_sim* s) { return s ? s->bytes : 0; }
 
 int ce_kernel_in_use(const ce_sim* s) { return s ? s->kernel : CE_KERNEL_GENERIC; }
 
+int ce_resident_in_use(const ce_sim* s) { return s && s->res.blocks > 0 ? 1 : 0; }
+
 int ce_replan(ce_sim* s, int rows, int stages, int zchunks) {
   g_err.clear();
   int rc = check_sim(s, "ce_replan");
