@@ -109,6 +109,13 @@ extern "C" {
                                         that never arrive, so its bounded waits run
                                         out (~0.5 ms) and each launch latches
                                         CE_ETIMEOUT; no GPU fault is involved     */
+#define CE_FLAG_TEST_WAIT_STALL   4  /* failure-detection tests only: in the
+                                        handle's first launch of the resident
+                                        kernel, or of the 3D FP64 kernel in its
+                                        start-up, the blocks or warps wait for one
+                                        more than there are, until the bounded wait
+                                        runs out (~0.5 ms) and the launch latches
+                                        CE_ETIMEOUT                               */
 
 /* Device allocator hooks (optional).  alloc returns a device pointer of at
  * least `bytes` (256-byte aligned) usable on `stream`, or NULL; release

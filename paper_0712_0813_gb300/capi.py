@@ -22,6 +22,7 @@ CE_VEL_SYNC, CE_VEL_STAGGERED = 0, 1
 CE_KERNEL_AUTO, CE_KERNEL_GENERIC, CE_KERNEL_SWEEP, CE_KERNEL_ROWS, CE_KERNEL_PLANES = 0, 1, 2, 3, 4
 CE_FLAG_ALLOW_UNSTABLE_DT = 1
 CE_FLAG_TEST_TMA_STALL = 2
+CE_FLAG_TEST_WAIT_STALL = 4
 
 ALLOC_FN = ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p, ctypes.c_void_p)
 RELEASE_FN = ctypes.CFUNCTYPE(None, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p, ctypes.c_void_p)

@@ -48,6 +48,7 @@ constexpr int kGraphSteps = 32;   // steps per captured CUDA graph (even: keeps 
 constexpr int kResidentCounterWords = 64;   // the counter has 256 bytes of its own
 constexpr int kResidentSteps = 4096;   // most steps of one resident launch
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz: bound of every device-side wait
+constexpr long long kStallCycles = 1LL << 20;    // the same in launches that a test makes wait
 
 }  // namespace
 
@@ -143,7 +144,7 @@ ce::StepArgs<T> make_step_args(const ce_sim* s, int in, bool half_kick) {
   a.update_scalars = (s->cfg.expansion && !half_kick) ? 1 : 0;
   a.in_slot = in;
   const bool stall = (s->cfg.flags & CE_FLAG_TEST_TMA_STALL) != 0;
-  a.wait_cycles = stall ? (1LL << 20) : kWaitCycles;
+  a.wait_cycles = stall ? kStallCycles : kWaitCycles;
   a.missing_tx = stall ? 16u : 0u;
   a.sc_in = &s->aux->slot[in];
   a.sc_out = &s->aux->slot[in ^ 1];
@@ -163,8 +164,15 @@ void fx_spacing(const ce_sim* s, Args& a) {
   a.source = ce::source_weights(dx, s->S);
 }
 
+// Whether this launch is the one that CE_FLAG_TEST_WAIT_STALL asks for.
+bool take_stall(ce_sim* s) {
+  const bool on = (s->cfg.flags & CE_FLAG_TEST_WAIT_STALL) != 0;
+  s->cfg.flags &= ~CE_FLAG_TEST_WAIT_STALL;
+  return on;
+}
+
 template <typename T>
-cudaError_t launch_one_step(const ce_sim* s, int in, bool half_kick) {
+cudaError_t launch_one_step(const ce_sim* s, int in, bool half_kick, bool stall) {
   if (s->kernel == CE_KERNEL_ROWS && !half_kick) return ce::rows_launch(s->rows, in, s->stream);
   ce::StepArgs<T> a = make_step_args<T>(s, in, half_kick);
   if (s->kernel == CE_KERNEL_SWEEP) return ce::launch_step_sweep<T>(a, s->plan, s->stream);
@@ -173,15 +181,17 @@ cudaError_t launch_one_step(const ce_sim* s, int in, bool half_kick) {
                         : ce::launch_step_lines<T>(a, s->lines, s->stream);
   if constexpr (sizeof(T) == 8) {
     fx_spacing(s, a);
+    a.missing_tx = stall ? 1u : 0u;
+    if (stall) a.wait_cycles = kStallCycles;
     return ce::launch_step_fx(a, s->fx, s->stream);
   } else {
     return ce::launch_step_generic(a, s->generic_blocks, s->stream);
   }
 }
 
-cudaError_t step_once(const ce_sim* s, int in, bool half_kick) {
-  return s->prec == CE_F32 ? launch_one_step<float>(s, in, half_kick)
-                           : launch_one_step<double>(s, in, half_kick);
+cudaError_t step_once(const ce_sim* s, int in, bool half_kick, bool stall = false) {
+  return s->prec == CE_F32 ? launch_one_step<float>(s, in, half_kick, stall)
+                           : launch_one_step<double>(s, in, half_kick, stall);
 }
 
 // n steps of a small lattice by the resident kernel, from buffer set `in`.
@@ -211,10 +221,11 @@ cudaError_t launch_resident_steps(ce_sim* s, int in, int n) {
   }
   a.slot = s->aux->slot;
   a.counter = s->res_counter;
-  a.count0 = s->res_count;
+  const bool stall = take_stall(s);
+  a.count0 = s->res_count + (stall ? 1u : 0u);
   a.shares = reinterpret_cast<double*>(s->res_counter + kResidentCounterWords);
   a.status = &s->aux->status;
-  a.wait_cycles = kWaitCycles;
+  a.wait_cycles = stall ? kStallCycles : kWaitCycles;
   return ce::launch_resident(a, s->dims, s->nf, s->stream);
 }
 
@@ -615,7 +626,8 @@ int ce_set_fields(ce_sim* s, const double* f, const double* v, int mode, const c
     // start-up: sums over (f(0), u(0)) -> a'(0), a''(0) -> half kick
     e = run_diag(s, /*raw_u=*/1);
     if (e == cudaSuccess) e = ce::launch_init_scalars(s->aux, s->cur, s->cfg.expansion, s->cfg.dt, s->kappa2, s->stream);
-    if (e == cudaSuccess) e = step_once(s, s->cur, /*half_kick=*/true);
+    const bool stall = s->prec == CE_F64 && s->dims == 3 && take_stall(s);
+    if (e == cudaSuccess) e = step_once(s, s->cur, /*half_kick=*/true, stall);
     if (e != cudaSuccess) return cuda_fail(e, "ce_set_fields: start-up");
     s->cur ^= 1;
     s->t = 0.0;

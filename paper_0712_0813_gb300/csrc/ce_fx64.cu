@@ -77,8 +77,9 @@ __global__ void __launch_bounds__(32 * (RB + 2), FxRows<NF>::blocks)
   __shared__ __align__(8) uint64_t bar[2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
-    mbar_init(&bar[0], RB + 2);
-    mbar_init(&bar[1], RB + 2);
+    const uint32_t rows = RB + 2 + p.missing_tx;   // one more where a test makes the waits run out
+    mbar_init(&bar[0], rows);
+    mbar_init(&bar[1], rows);
     fence_mbar_init();
   }
   __syncthreads();
