@@ -37,7 +37,12 @@ constexpr int kFlush = 16;   // sites a thread sums in T before adding to its ru
 // chunk of z; 2D: 256 x-sites swept along a chunk of y; 1D: 256 threads x 16
 // sites, strided.  Along the sweep the neighbours stay in registers.  Chunks of 16
 // (their end planes, read twice, hit L2), shorter where that leaves blocks without
-// a task: there one thread's sweep is pure latency.  Warp strips with the y- and
+// a task: there one thread's sweep is pure latency.  FP64, whose arithmetic costs more
+// than its loads, takes 256 consecutive sites of a plane in 3D (no lanes idle past a
+// row's end), chunks down to one site, and skips warps without sites: ce_energy
+// with four fields at 33^3 took 64 us in 32 x 8 tiles and chunks of 4 (now 50; 48 before
+// the sweeps, with a thread a site), 101^3 394 (275; 376), 1D 4099 68 in chunks of 16 (30;
+// 34).  Warp strips with the y- and
 // x-neighbours in registers and a plane of loads in flight (the column kernel's
 // layout) need half the loads but 164 registers: 217 against 142 us at 256^3.
 struct DiagTasks {
@@ -46,18 +51,19 @@ struct DiagTasks {
   int64_t count;
 };
 
-DiagTasks diag_tasks(int dims, int64_t N, int64_t S, int blocks) {
+DiagTasks diag_tasks(int dims, bool f64, int64_t N, int64_t S, int blocks) {
   DiagTasks t{1, 1, kFlush, 0};
-  if (dims == 1) {
-    t.count = (S + kDiagThreads * kFlush - 1) / (kDiagThreads * kFlush);
-    return t;
+  const bool linear = dims == 3 && f64;
+  if (linear) t.nx = (int)((N * N + kDiagThreads - 1) / kDiagThreads);
+  else if (dims > 1) t.nx = (int)((N + (dims == 3 ? 31 : kDiagThreads - 1)) / (dims == 3 ? 32 : kDiagThreads));
+  if (dims == 3 && !linear) t.ny = (int)((N + kDiagWarps - 1) / kDiagWarps);
+  const int shortest = f64 ? 1 : (dims == 1 ? kFlush : 4);
+  const int want = f64 ? blocks : blocks / 2;
+  for (t.len = kFlush;; t.len /= 2) {
+    t.count = dims == 1 ? (S + (int64_t)kDiagThreads * t.len - 1) / ((int64_t)kDiagThreads * t.len)
+                        : (int64_t)t.nx * t.ny * ((N + t.len - 1) / t.len);
+    if (t.count >= want || t.len == shortest) return t;
   }
-  t.nx = (int)((N + (dims == 3 ? 31 : kDiagThreads - 1)) / (dims == 3 ? 32 : kDiagThreads));
-  t.ny = dims == 3 ? (int)((N + kDiagWarps - 1) / kDiagWarps) : 1;
-  for (t.len = kFlush; t.len > 4; t.len /= 2)
-    if ((int64_t)t.nx * t.ny * ((N + t.len - 1) / t.len) >= blocks / 2) break;
-  t.count = (int64_t)t.nx * t.ny * ((N + t.len - 1) / t.len);
-  return t;
 }
 
 // Per-launch scalars in the storage type.
@@ -266,9 +272,10 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 
       T part[NV];
 #pragma unroll
       for (int j = 0; j < NV; ++j) part[j] = T(0);
-      const int64_t s0 = task * (kDiagThreads * kFlush) + threadIdx.x;
+      const int64_t s0 = task * (kDiagThreads * (sizeof(T) == 8 ? tk.len : kFlush)) + threadIdx.x;
+      const int len = sizeof(T) == 8 ? tk.len : kFlush;
 #pragma unroll 4
-      for (int r = 0; r < kFlush; ++r) {
+      for (int r = 0; r < len; ++r) {
         const int64_t s = s0 + r * kDiagThreads;
         if (s >= p.S) break;
         T f[NF], w[NF], nb[NF][1][2];
@@ -289,26 +296,41 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 
     for (int64_t task = blockIdx.x; task < tk.count; task += gridDim.x) {
       // the lane's column: (x, y) in 3D, x in 2D; columns past the lattice's end
       // repeat its last one and add nothing
-      const int xs = (int)(task % tk.nx);
-      const int64_t rest = task / tk.nx;
+      // FP64: the chunks of a column group follow one another (a plane's last group, which
+      // may hold few sites, goes to blocks that have a task already)
+      const int64_t inner = sizeof(T) == 8 ? tk.count / tk.nx : tk.nx;
+      const int xs = (int)(sizeof(T) == 8 ? task / inner : task % inner);
+      const int64_t rest = sizeof(T) == 8 ? task % inner : task / inner;
       const int n = (int)N;                                    // sides below 2^17
       int x, y = 0, chunk;
-      if constexpr (DIMS == 3) {
-        x = xs * 32 + lane;
-        y = (int)(rest % tk.ny) * kDiagWarps + warp;
-        chunk = (int)(rest / tk.ny);
-      } else {
-        x = xs * kDiagThreads + threadIdx.x;
+      bool site;
+      if constexpr (DIMS == 3 && sizeof(T) == 8) {
+        const int at = xs * kDiagThreads + threadIdx.x;
+        site = at < n * n;
+        y = min(at, n * n - 1) / n;
+        x = min(at, n * n - 1) - y * n;
         chunk = (int)rest;
+      } else {
+        if constexpr (DIMS == 3) {
+          x = xs * 32 + lane;
+          y = (int)(rest % tk.ny) * kDiagWarps + warp;
+          chunk = (int)(rest / tk.ny);
+        } else {
+          x = xs * kDiagThreads + threadIdx.x;
+          chunk = (int)rest;
+        }
+        site = x < n && y < n;
+        x = min(x, n - 1);
+        y = min(y, n - 1);
       }
-      const bool site = x < n && y < n;
-      x = min(x, n - 1);
-      y = min(y, n - 1);
       // offsets in a plane, added to the plane's (uniform) base
       const uint32_t o = (uint32_t)y * (uint32_t)n + x;
       const uint32_t oxp = x == n - 1 ? o - (n - 1) : o + 1, oxm = x == 0 ? o + (n - 1) : o - 1;
-      const uint32_t oyp = y == n - 1 ? o - (n - 1) * n : o + n, oym = y == 0 ? o + (n - 1) * n : o - n;
-      const int z0 = chunk * tk.len, z1 = min(z0 + tk.len, n);
+      const uint32_t column = (uint32_t)(n - 1) * (uint32_t)n;   // used in 3D only, where it fits
+      const uint32_t oyp = y == n - 1 ? o - column : o + n, oym = y == 0 ? o + column : o - n;
+      const int z0 = chunk * tk.len;
+      int z1 = min(z0 + tk.len, n);
+      if constexpr (sizeof(T) == 8) z1 = __any_sync(0xffffffffu, site) ? z1 : z0;   // no site: nothing to sum
       T fm[NF], fc[NF], part[NV];
 #pragma unroll
       for (int i = 0; i < NF; ++i) {
@@ -453,7 +475,7 @@ cudaError_t launch_diag_dims(const DiagArgs<T>& a, int cap, cudaStream_t st) {
     }
   }
   cap = std::min(cap, per_sm * sm_count(-1));
-  const DiagTasks tk = diag_tasks(DIMS, a.N, a.S, cap);
+  const DiagTasks tk = diag_tasks(DIMS, sizeof(T) == 8, a.N, a.S, cap);
   const int blocks = (int)std::min<int64_t>(tk.count, cap);
   k_diag<T, NF, DIMS><<<blocks, kDiagThreads, 0, st>>>(a, tk);
   return cudaGetLastError();
