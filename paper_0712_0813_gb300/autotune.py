@@ -118,7 +118,7 @@ def load(path: str):
             _cache[k] = TuneResult(v["tile_rows"], v["stages"], v["zchunks"], v["ms_per_step"])
 
 
-def autotune_batch(sims, *, candidates=(32, 64, 128, 256), occupancies=(0,), steps: int = 20,
+def autotune_batch(sims, *, candidates=(16, 32, 64, 128, 256), occupancies=(0,), steps: int = 20,
                    warmup: int = 4, stream=None) -> dict:
     """Pick the batched kernel's item length (sites per item along the sweep
     axis) and, optionally, a cap on resident CTAs per SM for a set of handles:
