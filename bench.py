@@ -835,7 +835,9 @@ def main():
             "scaling": "weak", "vs_baseline": None, "dtype": args.precision, "data": "synthetic",
             "config": {"workload": w["name"], "N": w["N"], "fields": w["nf"], "expansion": w["expansion"],
                        "dt": w["dt"], "L": w["L"], "precision": args.precision,
-                       "storage": "fields+velocities " + args.precision + ", global sums and a(t) f64",
+                       "storage": "fields+velocities " + args.precision + (", global sums f64 over pairs of f32 in a block"
+                                                                           if args.precision == "f32" else
+                                                                           ", global sums f64") + ", a(t) f64",
                        "kernel": kernel, "sweep_plan": {"tile_rows": plan[0], "stages": plan[1],
                                                          "zchunks": plan[2]},
                        "autotune": tune_info,

@@ -59,8 +59,9 @@ extern "C" {
 
 /* ---- precision ------------------------------------------------------- */
 #define CE_F64 0          /* fields, velocities and arithmetic in FP64       */
-#define CE_F32 1          /* fields and velocities in FP32; global sums and
-                             a, a', a'' in FP64                              */
+#define CE_F32 1          /* fields and velocities in FP32, a thread's sums of a
+                             few sites too; global sums in pairs of floats
+                             (48 bits) or FP64; a, a', a'' in FP64           */
 
 /* ---- velocity conventions for ce_set_fields / ce_get_fields ----------- */
 #define CE_VEL_SYNC      0  /* v = u(t) = f'(t) - (a'/a) f(t), synchronised
@@ -201,7 +202,8 @@ int ce_step(ce_sim* sim, int64_t n);
 int ce_synchronize(ce_sim* sim);
 
 /* Per-field mean <f_i> and population variance <(f_i - <f_i>)^2> at the
- * current integer time, FP64 sums.  Sec. II leaves the choice of outputs to
+ * current integer time, summed in FP64 or, FP32 handles, in pairs of floats (48
+ * bits) over partials of up to 16 sites.  Sec. II leaves the choice of outputs to
  * the run's parameters; per-field means and population variances are the
  * library's reading of the basic field statistics such a run writes out.
  * mean, var: host arrays of nf doubles, owned by the caller.  Synchronises.

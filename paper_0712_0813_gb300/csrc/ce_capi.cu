@@ -444,7 +444,7 @@ int ce_create(const ce_config* cfg, ce_sim** out) {
   // column kernel (3D) or the line-sweep kernel (2D) for odd and small sides,
   // else (1D lattices, small 2D sides) the generic kernel.  FP64, which GB300's
   // two FP64 lanes per clock and SM would bound: the kernels that form the force
-  // in integers (ce_fx64.cu, under CE_KERNEL_GENERIC; 256^3: 596 us against 1141
+  // in integers (ce_fx64.cu, under CE_KERNEL_GENERIC; 256^3: 616 us against 1141
   // for the tuned z-sweep kernel and 2967 at 288^3 for the row kernel), unless the
   // caller gave z-sweep plan hints.
   const bool sweep_hinted = cfg->tile_rows != 0 || cfg->stages != 0 || cfg->zchunks != 0;

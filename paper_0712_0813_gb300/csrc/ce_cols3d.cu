@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kColThreads, MB) k_step_cols(const StepArgs<T>
       y = y < 0 ? y + (int)N : y;
       y = y >= N ? y - (int)N : y;
       y = y >= N ? y % (int)N : y;                 // N < TY + 1: several wraps
-      ry[k] = (uint32_t)(y * (int)N + (int)xs) * (uint32_t)sizeof(T);   // N^3 <= 2^34: below 2^25
+      ry[k] = (uint32_t)(y * (int)N + (int)xs) * (uint32_t)sizeof(T);   // N^3 <= 2^34: below 2^26
     }
     const T c = (T)p.sc_in->c;
     const T dd = p.dt_drift, kk = p.dt_kick, idx2 = p.inv_dx2;

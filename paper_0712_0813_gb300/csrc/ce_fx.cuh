@@ -128,7 +128,7 @@ CE_FX_HD Fx from_double(double x) {
   return r;
 }
 
-// The double an Fx came from, bit for bit.
+// The double an Fx came from (0.0 for -0.0, else bit for bit).
 CE_FX_HD double to_double(const Fx& x) {
   const int64_t s = x.m >> 63;
   const int64_t frac = ((x.m ^ s) - s) >> 5;

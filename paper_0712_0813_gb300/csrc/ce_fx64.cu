@@ -9,18 +9,19 @@
 // What bounds it.  GB300 has two FP64 lanes per clock and SM, so the step in FP64
 // (a pass for g, a pass for the stencil, 32 operations a site with two fields) ran
 // at 0.85 of that pipe and 0.15 of HBM.  Here 10.2 FP64 operations a site remain
-// (256^3 by ncu, halo lanes included; half of that pipe) among 782 instructions, most
-// of them integer.  596 us a step at 256^3 (two passes: 1058), 30.9 ms at 1024^3 (67):
-// bound by issue and its latency, 0.60 of the issue slots with 17 warps an SM (96
-// registers a thread), beside 0.27 of HBM.
+// (256^3 by ncu, halo lanes included; half of that pipe) among 835 instructions, most
+// of them integer.  616 us a step at 256^3 (two passes: 1058; 596 with 782 instructions
+// when the model force was still cut to the unit of the fields): bound by issue and its
+// latency, 0.62 of the issue slots with 17 warps an SM (96 registers a thread), beside
+// 0.26 of HBM.
 //
-// Layout.  3D: the column kernel's (ce_cols3d.cu): a warp owns 30 x-sites by TY
-// rows and sweeps a chunk of z; lane l holds column x0 - 1 + l, so lanes 0 and
-// nx + 1 carry the x-halo and x-neighbours come by shuffles; y-neighbours are the
-// lane's own registers, z-neighbours the planes before and after.  Each plane's
-// values are converted to integers once, when g is formed.  2D: the same with one
-// row per lane, sweeping y.  1D: one strip of 30 sites at a time, no sweep.
-// Any side, no alignment, no shared memory in the sweep.
+// Layout.  A warp holds a strip of 30 x-sites, lane l the column x0 - 1 + l, so lanes 0
+// and nx + 1 carry the x-halo and x-neighbours come by shuffles.  3D: a block of RB + 2
+// warps, one row each, sweeps a chunk of z; rows above and below are read from a ring of
+// planes in shared memory, z-neighbours are the lane's own registers.  2D: a warp sweeps
+// a chunk of y by itself, y-neighbours in registers.  1D: one strip at a time, no sweep.
+// Each plane's values are converted to integers once, when g is formed.  Any side, no
+// alignment.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>

@@ -69,7 +69,9 @@ __global__ void k_shifted_copy(const T* __restrict__ f, T* __restrict__ out, int
     out[k] = f[k] - shift;
 }
 
-// floor(sqrt(x)) for 0 <= x < 2^34.
+// floor(sqrt(x)) for 0 <= x < 2^62: the float root is within 2^-23 of it, which the loops
+// make good (no step or one below x = 2^46; lattices end at sides of 2^34 in 1D, where a
+// bin's squares reach 2^62).
 __device__ __forceinline__ int isqrt(int64_t x) {
   int s = (int)sqrtf((float)x);
   while ((int64_t)s * s > x) --s;
@@ -365,7 +367,7 @@ SpectrumWork* find_work(const ce_sim* s, bool create) {
 }
 
 // Partial histograms a handle's work buffers hold.
-int spectrum_parts(const ce_sim* s) { return s->dims == 1 ? kBinChunks : kBinParts; }
+int spectrum_parts(const ce_sim* s) { return s->dims == 1 ? 1 : kBinParts; }
 
 constexpr char kMagic[8] = {'C', 'E', 'G', 'R', 'I', 'D', '0', '1'};
 

@@ -3,7 +3,7 @@
 // A lattice of some 10^5 sites takes a few microseconds a step whatever its
 // kernel: a launch, the first loads, the block sums, and the last block's tail (sum
 // of the partials, a', the end of the grid) follow one another.  Here the lattice
-// stays in the registers of one block per SM for all the steps of a ce_step call.
+// stays in the shared memory of at most one block per SM for the steps of a ce_step call.
 // Each block owns a brick of the lattice; per step it
 //   1. waits until every block has published the last step (a counter),
 //   2. loads f and w of its halo from L2, while one warp sums the blocks' shares of
