@@ -82,7 +82,7 @@ extern "C" {
                                one cooperative launch with up to a block on every
                                SM.  FP64: to 450000 sites in 3D, 600000 else.
                                FP32 with expansion and two fields or more: sites
-                               x fields to 524288 in 3D, 2000000 in 2D, 150000
+                               x fields to 524288 in 3D, 2200000 in 2D, 150000
                                sites in 1D.  FP32 without expansion: sites x
                                fields to 65536 in 3D, 360000 to 700000 sites in
                                2D.  One handle at a time is what it is fastest

@@ -216,7 +216,7 @@ inline bool resident_takes(int dims, int64_t S, int nf, bool f64, bool expansion
   if (f64) return S <= (dims == 3 ? 450000 : 600000);
   if (!expansion) return dims == 3 ? S * nf <= 65536 : dims == 2 && S >= 360000 && S <= 700000;
   if (dims == 1) return S <= 150000;
-  return S * nf <= (dims == 3 ? 524288 : 2000000);
+  return S * nf <= (dims == 3 ? 524288 : 2200000);
 }
 
 }  // namespace plan

@@ -43,7 +43,7 @@ def test_lattices_of_several_sizes_side_by_side(gpu_capi, precision, dims, sizes
 ROUTES = [(3, 76, 2, "f64", True, True), (3, 77, 2, "f64", True, False), (2, 774, 1, "f64", False, True),
           (2, 775, 1, "f64", False, False), (1, 600000, 2, "f64", True, True), (1, 600001, 2, "f64", True, False),
           (3, 64, 2, "f32", True, True), (3, 65, 2, "f32", True, False), (3, 50, 4, "f32", True, True),
-          (3, 51, 4, "f32", True, False), (2, 1000, 2, "f32", True, True), (2, 1001, 2, "f32", True, False),
+          (3, 51, 4, "f32", True, False), (2, 1048, 2, "f32", True, True), (2, 1049, 2, "f32", True, False),
           (1, 150000, 2, "f32", True, True), (1, 150001, 2, "f32", True, False), (3, 16, 1, "f32", True, False),
           (3, 32, 2, "f32", False, True), (3, 33, 2, "f32", False, False), (2, 599, 2, "f32", False, False),
           (2, 600, 2, "f32", False, True), (2, 836, 4, "f32", False, True), (2, 837, 4, "f32", False, False),
