@@ -143,11 +143,13 @@ __device__ __forceinline__ int64_t grid_blocks() {
 // runs once per block or per step is written for few FP64 instructions: the end of
 // a block and of a launch below took ~6 us of a step, the launch gap ~2.
 
-// hi + lo += x: the addition's rounding error (Knuth's TwoSum, exact) joins lo.
+// hi + lo += x: the addition's rounding error (Knuth's TwoSum, exact) joins lo.  Intrinsics,
+// which the compiler does not contract with a product that x may be: else what is added
+// would depend on the code around.
 __device__ __forceinline__ void add_to(float& hi, float& lo, float x) {
-  const float s = hi + x;
-  const float b = s - hi;
-  lo += (hi - (s - b)) + (x - b);
+  const float s = __fadd_rn(hi, x);
+  const float b = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
   hi = s;
 }
 

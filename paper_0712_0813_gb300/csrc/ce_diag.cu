@@ -10,11 +10,10 @@
 //
 // The pass reads f and w once (2 NF x sizeof(T) per site).  For FP32 storage HBM
 // bounds it, provided the FP64 pipe (two lanes per clock and SM: 64 cycles a warp
-// instruction and scheduler) stays out of it: a thread's partials stay in FP32 for
-// at most 16 sites and are then added, with the addition's rounding error kept
-// (add_to), to float pairs of 48 bits, which the lanes add the same way; only the
-// warps' sums become FP64.  The partials' own rounding (2^-24 over 16 sites) is what
-// limits the sums, as when they went to FP64 accumulators.  That flush, as a counter
+// instruction and scheduler) stays out of it: a thread's partials over at most 16
+// sites (in FP32, on smaller lattices in float pairs: Partials) are added, with the
+// addition's rounding error kept (add_to), to float pairs of 48 bits, which the lanes
+// add the same way; only the warps' sums become FP64.  That flush, as a counter
 // test inside the site loop, was if-converted into 9 conversions and 9 FP64
 // additions a site (256^3, two fields: 606 us where the bytes take 40), and as a
 // loop of its own still took 202 us, half of it the warps' FP64 shuffle sums.
@@ -87,15 +86,45 @@ __device__ __forceinline__ DiagScalars<T> diag_scalars(const DiagArgs<T>& p) {
   return k;
 }
 
+// A thread's sums over the sites of a task, up to kFlush of them: in T, or in pairs of
+// floats (FP32 lattices below kPairSites).  Few sites leave few sums for their rounding to
+// average over: in plain FP32 V of 1D 65536 was off by 1.1e-9 where FP64 sums of the sites
+// give 2.8e-10 and the pairs 2.3e-10.  Large lattices keep 16 sites in FP32 (256^3: V 3e-10
+// either way, 138 us against 181 with pairs; 1D 2 M 49 us with, 44 without); the
+// squares of a site's gradient are added before they join the sum, without which G was
+// off by 1.6e-8 (3.2e-9).
+constexpr int64_t kPairSites = 5000000;
+
+template <typename T, int NV, bool PAIRS>
+struct Partials {
+  T v[NV];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) v[j] = T(0);
+  }
+  __device__ __forceinline__ void add(int j, T x) { v[j] += x; }
+  __device__ __forceinline__ void add_product(int j, T x, T y) { v[j] = fmaT(x, y, v[j]); }
+};
+template <int NV>
+struct Partials<float, NV, true> {
+  float v[NV], lo[NV];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) v[j] = lo[j] = 0.f;
+  }
+  __device__ __forceinline__ void add(int j, float x) { add_to(v[j], lo[j], x); }
+  __device__ __forceinline__ void add_product(int j, float x, float y) { add(j, x * y); }
+};
+
 // One site's terms added to part: [K_i (NF)][G_i (NF)][V][f_i - f_i(0) (NF)]
 // [(f_i - f_i(0))^2 (NF)].  nb[d][0] / nb[d][1]: the neighbours at +e_d / -e_d.
-template <typename T, int NF, int DIMS>
+template <bool PAIRS, typename T, int NF, int DIMS>
 __device__ __forceinline__ void diag_site(const DiagScalars<T>& k, int raw_u, const T (&f)[NF], const T (&w)[NF],
                                           const T (&nb)[NF][DIMS][2], const T (&shift)[NF],
-                                          T (&part)[4 * NF + 1]) {
+                                          Partials<T, 4 * NF + 1, PAIRS>& part) {
   T dv[NF], vs;
   model_dv<T, NF>(f, k.q, dv, vs);
-  part[2 * NF] += vs;
+  part.add(2 * NF, vs);
 #pragma unroll
   for (int i = 0; i < NF; ++i) {
     T lap = T(0);
@@ -108,10 +137,17 @@ __device__ __forceinline__ void diag_site(const DiagScalars<T>& k, int raw_u, co
 #pragma unroll
       for (int d = 0; d < DIMS; ++d) lap += (nb[i][d][0] + nb[i][d][1]) - T(2) * f[i];
     }
+    if constexpr (sizeof(T) == 8) {
 #pragma unroll
-    for (int d = 0; d < DIMS; ++d) {
-      const T df = nb[i][d][0] - f[i];
-      part[NF + i] = fmaT(df, df, part[NF + i]);
+      for (int d = 0; d < DIMS; ++d) part.add_product(NF + i, nb[i][d][0] - f[i], nb[i][d][0] - f[i]);
+    } else {
+      T g2 = T(0);
+#pragma unroll
+      for (int d = 0; d < DIMS; ++d) {
+        const T df = nb[i][d][0] - f[i];
+        g2 = fmaT(df, df, g2);
+      }
+      part.add(NF + i, g2);
     }
     T u = w[i];
     if (!raw_u) {
@@ -119,10 +155,10 @@ __device__ __forceinline__ void diag_site(const DiagScalars<T>& k, int raw_u, co
       const T F = fmaT(lap, k.idx2, -dv[i]) + k.sterm * f[i];
       u = fmaT(-k.half_dt, F, vh) - k.h * f[i];
     }
-    part[i] = fmaT(T(0.5) * u, u, part[i]);
+    part.add_product(i, T(0.5) * u, u);
     const T df = f[i] - shift[i];
-    part[2 * NF + 1 + i] += df;
-    part[3 * NF + 1 + i] = fmaT(df, df, part[3 * NF + 1 + i]);
+    part.add(2 * NF + 1 + i, df);
+    part.add_product(3 * NF + 1 + i, df, df);
   }
 }
 
@@ -138,9 +174,9 @@ struct RunningSums<double, NV> {
 #pragma unroll
     for (int j = 0; j < NV; ++j) v[j] = 0.0;
   }
-  __device__ __forceinline__ void add(const double (&part)[NV], double*) {
+  __device__ __forceinline__ void add(const Partials<double, NV, false>& part, double*) {
 #pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] += part[j];
+    for (int j = 0; j < NV; ++j) v[j] += part.v[j];
   }
   __device__ __forceinline__ double warp_total(int j) { return warp_sum(v[j]); }
 };
@@ -151,16 +187,24 @@ struct RunningSums<float, NV> {
 #pragma unroll
     for (int j = 0; j < NV; ++j) hi[j] = lo[j] = 0.f;
   }
-  __device__ __forceinline__ void add(const float (&part)[NV], double* big) {
+  template <bool PAIRS>
+  __device__ __forceinline__ void add(const Partials<float, NV, PAIRS>& part, double* big) {
     bool fits = true;
 #pragma unroll
-    for (int j = 0; j < NV; ++j) fits = fits && fabsf(part[j]) < 0x1p100f;
+    for (int j = 0; j < NV; ++j) fits = fits && fabsf(part.v[j]) < 0x1p100f;
     if (__all_sync(0xffffffffu, fits)) {   // every lane of the warp is here
 #pragma unroll
-      for (int j = 0; j < NV; ++j) add_to(hi[j], lo[j], part[j]);
+      for (int j = 0; j < NV; ++j) {
+        add_to(hi[j], lo[j], part.v[j]);
+        if constexpr (PAIRS) lo[j] += part.lo[j];
+      }
     } else {
 #pragma unroll
-      for (int j = 0; j < NV; ++j) atomicAdd(big + j, (double)part[j]);
+      for (int j = 0; j < NV; ++j) {
+        double x = part.v[j];
+        if constexpr (PAIRS) x += isfinite(part.lo[j]) ? (double)part.lo[j] : 0.0;
+        atomicAdd(big + j, x);
+      }
     }
   }
   __device__ __forceinline__ double warp_total(int j) {
@@ -252,7 +296,7 @@ __device__ __forceinline__ void diag_finish(const DiagArgs<T>& p, RunningSums<T,
   if (threadIdx.x == 0) p.aux->counter_diag = 0u;
 }
 
-template <typename T, int NF, int DIMS>
+template <typename T, int NF, int DIMS, bool PAIRS>
 __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 1) k_diag(const DiagArgs<T> p, const DiagTasks tk) {
   constexpr int NV = 4 * NF + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -269,9 +313,8 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 
   for (int i = 0; i < NF; ++i) shift[i] = p.f[i][0];
   if constexpr (DIMS == 1) {
     for (int64_t task = blockIdx.x; task < tk.count; task += gridDim.x) {
-      T part[NV];
-#pragma unroll
-      for (int j = 0; j < NV; ++j) part[j] = T(0);
+      Partials<T, NV, PAIRS> part;
+      part.clear();
       const int64_t s0 = task * (kDiagThreads * (sizeof(T) == 8 ? tk.len : kFlush)) + threadIdx.x;
       const int len = sizeof(T) == 8 ? tk.len : kFlush;
 #pragma unroll 4
@@ -286,7 +329,7 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 
           nb[i][0][0] = __ldg(p.f[i] + (s == N - 1 ? 0 : s + 1));
           nb[i][0][1] = __ldg(p.f[i] + (s == 0 ? N - 1 : s - 1));
         }
-        diag_site<T, NF, 1>(k, raw_u, f, w, nb, shift, part);
+        diag_site<PAIRS, T, NF, 1>(k, raw_u, f, w, nb, shift, part);
       }
       __syncwarp();
       acc.add(part, big);
@@ -331,14 +374,14 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 
       const int z0 = chunk * tk.len;
       int z1 = min(z0 + tk.len, n);
       if constexpr (sizeof(T) == 8) z1 = __any_sync(0xffffffffu, site) ? z1 : z0;   // no site: nothing to sum
-      T fm[NF], fc[NF], part[NV];
+      T fm[NF], fc[NF];
+      Partials<T, NV, PAIRS> part;
+      part.clear();
 #pragma unroll
       for (int i = 0; i < NF; ++i) {
         fm[i] = __ldg(p.f[i] + (z0 == 0 ? n - 1 : z0 - 1) * plane + o);
         fc[i] = __ldg(p.f[i] + z0 * plane + o);
       }
-#pragma unroll
-      for (int j = 0; j < NV; ++j) part[j] = T(0);
       constexpr int kUnroll = sizeof(T) == 8 ? 1 : (NF <= 2 ? 2 : 4);
 #pragma unroll kUnroll
       for (int z = z0; z < z1; ++z) {
@@ -358,17 +401,14 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 && NF <= 2 ? 4 : 
           nb[i][DIMS - 1][0] = fn[i];
           nb[i][DIMS - 1][1] = fm[i];
         }
-        diag_site<T, NF, DIMS>(k, raw_u, fc, w, nb, shift, part);
+        diag_site<PAIRS, T, NF, DIMS>(k, raw_u, fc, w, nb, shift, part);
 #pragma unroll
         for (int i = 0; i < NF; ++i) {
           fm[i] = fc[i];
           fc[i] = fn[i];
         }
       }
-      if (!site) {   // the whole warp takes part in the addition
-#pragma unroll
-        for (int j = 0; j < NV; ++j) part[j] = T(0);
-      }
+      if (!site) part.clear();   // the whole warp takes part in the addition
       __syncwarp();
       acc.add(part, big);
     }
@@ -409,9 +449,8 @@ __global__ void __launch_bounds__(kDiagThreads, NF <= 2 ? 4 : 2) k_start_sums(co
   const float q[3] = {(float)p.q[0], (float)p.q[1], (float)p.q[2]};
   const int64_t groups = ((p.S + stride - 1) / stride + kFlush - 1) / kFlush;
   for (int64_t g = 0; g < groups; ++g) {
-    float part[NV];
-#pragma unroll
-    for (int j = 0; j < NV; ++j) part[j] = 0.f;
+    Partials<float, NV, false> part;
+    part.clear();
 #pragma unroll 4
     for (int r = 0; r < kFlush; ++r) {
       if (s >= p.S) break;
@@ -430,11 +469,11 @@ __global__ void __launch_bounds__(kDiagThreads, NF <= 2 ? 4 : 2) k_start_sums(co
           const float df = __ldg(p.f[i] + up[d]) - f[i];
           g2 = fmaf(df, df, g2);
         }
-        part[i] = fmaf(0.5f * u, u, part[i]);
-        part[NF + i] += g2;
+        part.v[i] = fmaf(0.5f * u, u, part.v[i]);
+        part.v[NF + i] += g2;
       }
       model_dv<float, NF>(f, q, dv, vs);
-      part[2 * NF] += vs;
+      part.v[2 * NF] += vs;
       s += stride;
       if constexpr (DIMS >= 2) {   // in range again after one subtraction each
         x += dx;
@@ -459,26 +498,32 @@ __global__ void __launch_bounds__(kDiagThreads, NF <= 2 ? 4 : 2) k_start_sums(co
 }
 
 // A grid that is resident as a whole (at most `cap` blocks): tasks are strided.
-template <typename T, int NF, int DIMS>
-cudaError_t launch_diag_dims(const DiagArgs<T>& a, int cap, cudaStream_t st) {
+template <typename T, int NF, int DIMS, bool PAIRS>
+cudaError_t launch_diag_kernel(const DiagArgs<T>& a, int cap, cudaStream_t st) {
   int per_sm = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_diag<T, NF, DIMS>, kDiagThreads, 0) != cudaSuccess ||
-      per_sm < 1) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_diag<T, NF, DIMS, PAIRS>, kDiagThreads, 0) !=
+          cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     per_sm = 1;
   }
+  cap = std::min(cap, per_sm * sm_count(-1));
+  const DiagTasks tk = diag_tasks(DIMS, sizeof(T) == 8, a.N, a.S, cap);
+  const int blocks = (int)std::min<int64_t>(tk.count, cap);
+  k_diag<T, NF, DIMS, PAIRS><<<blocks, kDiagThreads, 0, st>>>(a, tk);
+  return cudaGetLastError();
+}
+
+template <typename T, int NF, int DIMS>
+cudaError_t launch_diag_dims(const DiagArgs<T>& a, int cap, cudaStream_t st) {
   if constexpr (sizeof(T) == 4) {
     if (a.raw_u && a.expansion) {
       const int blocks = (int)std::min<int64_t>((a.S + kDiagThreads - 1) / kDiagThreads, cap);
       k_start_sums<NF, DIMS><<<blocks, kDiagThreads, 0, st>>>(a);
       return cudaGetLastError();
     }
+    if (a.S < kPairSites) return launch_diag_kernel<T, NF, DIMS, true>(a, cap, st);
   }
-  cap = std::min(cap, per_sm * sm_count(-1));
-  const DiagTasks tk = diag_tasks(DIMS, sizeof(T) == 8, a.N, a.S, cap);
-  const int blocks = (int)std::min<int64_t>(tk.count, cap);
-  k_diag<T, NF, DIMS><<<blocks, kDiagThreads, 0, st>>>(a, tk);
-  return cudaGetLastError();
+  return launch_diag_kernel<T, NF, DIMS, false>(a, cap, st);
 }
 
 template <typename T, int NF>

@@ -55,11 +55,13 @@ int scratch_for_device(int dev, double** out) {
   return CE_OK;
 }
 
-// hi + lo += x: the addition's rounding error (Knuth's TwoSum, exact) joins lo.
+// hi + lo += x: the addition's rounding error (Knuth's TwoSum, exact) joins lo.  Intrinsics,
+// which the compiler does not contract with a product that x may be: else what is added
+// would depend on the code around.
 __device__ __forceinline__ void add_to(float& hi, float& lo, float x) {
-  const float s = hi + x;
-  const float b = s - hi;
-  lo += (hi - (s - b)) + (x - b);
+  const float s = __fadd_rn(hi, x);
+  const float b = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
   hi = s;
 }
 
